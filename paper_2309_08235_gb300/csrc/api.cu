@@ -268,8 +268,8 @@ void carve_ptrs(priest_loaded *h, char *b, const Carve &k, bool fp32, int z_iter
 }
 
 // PRIEST_NEIGHBOUR_LISTS=0 in the environment (read at every launch set-up)
-// makes the point-owner kernel screen every obstacle in every iteration
-// (comparisons); lists are on otherwise.
+// makes the point-owner kernel screen every time stamp in every iteration
+// (comparisons; bitwise the same results); lists are on otherwise.
 bool neighbour_lists()
 {
     const char *v = getenv("PRIEST_NEIGHBOUR_LISTS");
@@ -315,7 +315,8 @@ ProjParams<Real> proj_params(const priest_ctx *ctx, const priest_loaded *h, cons
     p.cB = h->cB;
     p.seg_len = h->seg_len;
     p.cost = make_cost<Real>(sh);
-    p.list_delta = neighbour_lists() ? Real(sh.list_delta) : Real(0);
+    p.list_delta = Real(sh.list_delta);
+    p.list_on = neighbour_lists() ? 1 : 0;
     p.list_grid = list_grid() ? 1 : 0;
     return p;
 }
@@ -385,6 +386,19 @@ void fill_result(const Shape &sh, const double *host_out, const double *host_mu,
     res->cost = host_out[sh.D + 1];
     res->c_aug = host_out[sh.D + 2];
     res->best_index = int(host_out[sh.D + 3]);
+}
+
+// Point-owner tilings of one persistent launch from all its samples; returns the
+// lanes per sample they share.
+int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles)
+{
+    size_t total = 0;
+    for (const Shape &sh : shapes) total += size_t(sh.N);
+    const int m = int((total + ctx->n_sm - 1) / ctx->n_sm);
+    int G = 16;
+    for (const Shape &sh : shapes) G = std::max(G, pts_group(sh, m));
+    for (size_t i = 0; i < shapes.size(); ++i) tiles[i] = pts_batch_tiling(shapes[i], G, m);
+    return G;
 }
 
 template ProjParams<float> proj_params<float>(const priest_ctx *, const priest_loaded *, const Tiling &);
@@ -562,14 +576,15 @@ template <typename Real>
 Tiling pick_tiling(priest_ctx *ctx, const Shape &sh, int N, ProjParams<Real> p, cudaStream_t st)
 {
     const Tiling model = choose_tiling<Real>(sh, N, ctx->n_sm);
-    if (!ctx->cfg.autotune) return model;
+    // the point-owner kernel has one tiling per shape (its sizes come from the SM's limits)
+    if (!ctx->cfg.autotune || model.kind == 1) return model;
     const std::vector<int> key = {int(sizeof(Real)), sh.dims, sh.nv, sh.nf, sh.n_p, sh.n_obs, sh.n_static,
                                   N, p.want_lambda, sh.use_bounds};
     load_tune_cache(ctx);
     auto it = ctx->tuned.find(key);
-    if (it != ctx->tuned.end()) {
+    if (it != ctx->tuned.end() && it->second.kind == 0) {
         Tiling t = it->second;
-        if (t.smem == 0) t.smem = t.kind == 1 ? pts_smem_bytes(sh, t.S, t.R) : project_smem_bytes<Real>(sh, t.S, t.C);
+        if (t.smem == 0) t.smem = project_smem_bytes<Real>(sh, t.S, t.C);
         return t;
     }
     std::vector<Tiling> cands = tiling_candidates<Real>(sh, N, ctx->n_sm);
@@ -1072,15 +1087,14 @@ std::vector<int> batch_class(const Shape &sh, int dbl)
 template <typename Real>
 Tiling batch_tiling_for(priest_ctx *ctx, const Shape &sh)
 {
+    const Tiling model = batch_tiling<Real>(sh);
+    if (model.kind == 1) return model;  // the point-owner kernel is not tuned
     auto it = ctx->tuned.find(batch_class(sh, sizeof(Real) == 8));
-    if (it == ctx->tuned.end()) return batch_tiling<Real>(sh);
+    if (it == ctx->tuned.end() || it->second.kind != 0) return model;
     Tiling t = it->second;
     t.S = std::max(1, std::min(t.S, sh.N));
-    t.smem = t.kind == 1 ? pts_smem_bytes(sh, t.S, t.R) : project_smem_bytes<Real>(sh, t.S, t.C);
-    if (t.smem > size_t(227) * 1024) return batch_tiling<Real>(sh);
-    // an entry from a cache file written for another CTA size
-    if (t.kind == 1 && (t.R != 2 || pts_threads(sh, t.S, 2) > pts_batch_threads(sh))) return batch_tiling<Real>(sh);
-    return t;
+    t.smem = project_smem_bytes<Real>(sh, t.S, t.C);
+    return t.smem > size_t(227) * 1024 ? model : t;
 }
 
 // shapes[i]: problem i's shape with the sample count of the launch; base[i]:
@@ -1098,7 +1112,7 @@ priest_status tune_batch(priest_ctx *ctx, int n, const std::vector<Shape> &shape
     {
         std::map<std::vector<int>, int> seen;
         for (int i = 0; i < n; ++i) {
-            if (shapes[i].N < 1) continue;
+            if (shapes[i].N < 1 || batch_tiling<Real>(shapes[i]).kind == 1) continue;
             const std::vector<int> key = batch_class(shapes[i], sizeof(Real) == 8);
             if (ctx->tuned.count(key) || seen.count(key)) continue;
             seen[key] = i;
@@ -1235,7 +1249,8 @@ priest_status batch_tiles(priest_ctx *ctx, const std::vector<Shape> &shapes, std
                 }
         }
     kind = all_pts ? 1 : 0;
-    R = all_pts ? tiles[0].R : 4;
+    R = 4;
+    if (all_pts) R = pts_batch_tiles(ctx, shapes, tiles);
     for (int i = 0; i < n; ++i)
         if (tiles[i].smem == 0 || tiles[i].kind != kind)
             return fail(ctx, PRIEST_ERR_INVALID, "problem too large for one CTA's shared memory");

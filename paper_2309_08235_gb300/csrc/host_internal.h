@@ -101,6 +101,9 @@ Carve carve(const Shape &sh, bool fp32, int z_iters, bool proj_buffers);
 // Points h's buffers into `base` laid out as k.
 void carve_ptrs(priest_loaded *h, char *base, const Carve &k, bool fp32, int z_iters, bool proj_buffers);
 
+// Point-owner tilings of one persistent launch; returns the lanes per sample.
+int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles);
+
 template <typename Real>
 ProjParams<Real> proj_params(const priest_ctx *ctx, const priest_loaded *h, const Tiling &t);
 SetupParams setup_params(const priest_ctx *ctx, const priest_loaded *h, bool plan_mode, int *status);

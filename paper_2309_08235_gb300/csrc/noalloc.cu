@@ -229,7 +229,7 @@ extern "C" priest_status priest_project_noalloc(const priest_config *cfg, const 
         p.xi_bar = xi_bar_dev; p.r_out = resid_dev; p.c1_out = cost_dev;
         p.cost = make_cost<float>(sh);
         p.list_delta = float(sh.list_delta);
-        p.list_grid = 1;
+        p.list_on = p.list_grid = 1;
         if (launch_project<float>(p, t, st) != cudaSuccess) return PRIEST_ERR_CUDA;
     } else {
         const Tiling t = choose_tiling<double>(sh, n, n_sm);

@@ -37,28 +37,25 @@ struct Shape {
     int N, n_proj, n_elite, D;
     int cost_kind;                          // c_1: 0 = sum |a|^2; 1 = BARN-style
     double w_acc, w_curv, w_path, curv_eps;
-    double list_delta;                      // neighbour-list margin: 3/4 of the mean of min(a_j, b_j)
-                                            // (0 without obstacles)
+    double list_delta;                      // neighbour-list margin (list_margin; 0 without obstacles)
 };
 
-// Neighbour-list margin of a problem: 3/4 of the mean of the obstacles'
-// smallest semi-axes (b_j = a_j in 2-D), 0 without obstacles (center:
-// n_obs x dims, semi: n_obs x 2).  Any positive margin gives bitwise the
-// same results; this one balanced list length against rebuild frequency on
-// the measured workloads (a margin of 0.5 to 1 mean semi-axis changed the
-// batched rate by under 2 %).  PRIEST_LIST_MARGIN=<multiple> replaces the
-// 3/4 (comparisons).  In dense scenes (64 obstacles or more) it is
-// capped so that a ball of radius (mean largest semi-axis + margin) holds
-// about two obstacle centres on average at the density of the centres'
-// bounding box, keeping the lists short of overflow; it stays at least a
-// tenth of the mean semi-axis.
+// Neighbour-list margin of a problem (center: n_obs x dims, semi: n_obs x 2), 0
+// without obstacles.  Any positive margin gives bitwise the same results; it
+// balances list length against rebuild frequency.  Many obstacles stiffen the
+// shared inverse (W = (I + rho (n_obs P^T P + ...))^-1), so the denser the scene
+// the slower its trajectories move: the margin is such that the ball of radius
+// (mean largest semi-axis + margin) holds 0.25 obstacle centres on average at
+// the density of the centres' bounding box, kept between 1/4 and 5/2 of the
+// mean smallest semi-axis; 3/2 of it below 16 obstacles.
+// PRIEST_LIST_MARGIN=<multiple> sets the multiple instead (comparisons).
 inline double list_margin_scale()
 {
     const char *v = getenv("PRIEST_LIST_MARGIN");
-    if (!v) return 0.75;
+    if (!v) return 0.0;
     char *end = nullptr;
     const double x = strtod(v, &end);
-    return (end != v && x > 0.0 && x < 1e6) ? x : 0.75;
+    return (end != v && x > 0.0 && x < 1e6) ? x : 0.0;
 }
 
 inline double list_margin(int dims, int n_obs, const double *center, const double *semi)
@@ -77,18 +74,16 @@ inline double list_margin(int dims, int n_obs, const double *center, const doubl
     }
     s /= n_obs;
     big /= n_obs;
-    double delta = list_margin_scale() * s;
-    if (n_obs >= 64) {
-        double vol = 1.0;
-        for (int ax = 0; ax < dims; ++ax) vol *= (hi[ax] - lo[ax]) + 2.0 * big;
-        const double rho = n_obs / vol, pi = 3.141592653589793;
-        // radius of the ball that holds two centres on average
-        const double r2 = dims == 2 ? __builtin_sqrt(2.0 / (pi * rho)) : __builtin_cbrt(1.5 / (pi * rho));
-        const double cap = r2 - big;
-        if (cap < delta) delta = cap;
-        if (delta < 0.1 * s) delta = 0.1 * s;
-    }
-    return delta;
+    const double scale = list_margin_scale();
+    if (scale > 0.0) return scale * s;
+    if (n_obs < 16) return 1.5 * s;
+    double vol = 1.0;
+    for (int ax = 0; ax < dims; ++ax) vol *= (hi[ax] - lo[ax]) + 2.0 * big;
+    const double rho = n_obs / vol, pi = 3.141592653589793, held = 0.25;
+    // radius of the ball that holds `held` centres on average
+    const double r = dims == 2 ? __builtin_sqrt(held / (pi * rho)) : __builtin_cbrt(0.75 * held / (pi * rho));
+    const double delta = r - big;
+    return delta < 0.25 * s ? 0.25 * s : delta > 2.5 * s ? 2.5 * s : delta;
 }
 
 // c_1 of the final pass (Alg. 1 cost): the point-to-point benchmark's
@@ -273,9 +268,9 @@ struct ProjParams {
     int N, K, S, C, WS, want_lambda, mode;  // mode 0: xi_in given; 1: xi = mu + L z; WS warps per sample
     int seg_len;                            // mode 1: samples per distribution (mu, Lc hold one per
                                             // segment of seg_len rows; 0 = a single distribution)
-    Real list_delta;                        // point-owner kernel: neighbour-list margin (0: screen every
-                                            // obstacle in every iteration)
-    int list_grid;                          // 1: list builds use the tables' static-obstacle grid
+    Real list_delta;                        // point-owner kernel: neighbour-list margin
+    int list_on;                            // 0: screen every time stamp in every iteration
+    int list_grid;                          // 1: screening uses the tables' static-obstacle grid
     CostParams<Real> cost;
     Real rho, vmax, amax, smin[3], smax[3];
     const Real *tab;
@@ -312,8 +307,8 @@ struct Tiling {
     int S;        // samples per CTA
     int C;        // obstacle chunks per CTA
     int threads;  // CTA size
-    int R;        // points per obstacle-loop item / per thread (template value)
-    int ws;       // warps per sample
+    int R;        // points per obstacle-loop item (chunked) / lanes per sample (point-owner): template values
+    int ws;       // warps per sample (chunked) / warps of the CTA that take samples (point-owner)
     size_t smem;  // dynamic shared memory bytes
     int kind = 0; // 0: chunked kernel (project_kernel.cuh); 1: point-owner FP32 kernel (project_pts.cuh)
 };
@@ -321,12 +316,12 @@ struct Tiling {
 // FP32 point-owner kernel (project_pts.cu): degree 10 with 5 free coefficients
 // (2-D, 3-D) or 7 (2-D).
 bool pts_supported(const Shape &sh);
-bool pts_span_ok(const Shape &sh, int R);
-bool pts_batch_ok(const Shape &sh);
-size_t pts_smem_bytes(const Shape &sh, int S, int R);
-int pts_threads(const Shape &sh, int S, int R);
-int pts_max_threads(int R);                 // largest CTA of the single-problem variants
-int pts_batch_threads(const Shape &sh);     // CTA of the persistent variant for sh
+size_t pts_smem_bytes(const Shape &sh, int G, int warps, int C);  // C warps per sample
+int pts_group(const Shape &sh, int samples_per_sm);    // lanes per sample (16 or 32)
+Tiling pts_tiling(const Shape &sh, int G, int warps);  // 32 / G samples per warp; smem 0: does not fit
+int pts_team_size(const Shape &sh, int samples_per_sm);  // warps per sample of a team, 0: no team
+Tiling pts_team_tiling(const Shape &sh, int teams, int C);  // teams of C warps, a sample each
+Tiling pts_batch_tiling(const Shape &sh, int G, int samples_per_sm);  // item of the persistent launch
 
 // Raises a kernel's dynamic shared-memory limit to `bytes` (the default limit
 // counts static shared memory too, so it is raised whenever more is asked
@@ -434,7 +429,8 @@ template <typename Real>
 cudaError_t launch_project(const ProjParams<Real> &p, const Tiling &t, cudaStream_t st);
 cudaError_t launch_project_pts(const ProjParams<float> &p, const Tiling &t, cudaStream_t st);
 cudaError_t launch_project_pts_batch(const ProjParams<float> *params, const int2 *items, int n_items, int *counter,
-                                     int dims, int nf, int R, int want_lambda, size_t smem, int grid, cudaStream_t st);
+                                     int dims, int nf, int G, int want_lambda, size_t smem, int grid,
+                                     cudaStream_t st);
 
 template <typename Real>
 Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm);

@@ -58,59 +58,35 @@ int samples_per_cta(int n_samples, int n_sm, int threads, int ws)
     return std::max(1, S);
 }
 
-bool pts_allowed();
-
-// Point-owner tiling (FP32, project_pts.cuh): S samples per CTA with R points
-// per thread; smem == 0 when the CTA does not fit.
-Tiling pts_tiling(const Shape &sh, int S, int R)
+// PRIEST_PROJECT_KERNEL=chunked in the environment keeps the FP32 projection
+// on the chunked kernel (comparisons).
+bool pts_allowed()
 {
-    Tiling t;
-    t.kind = 1;
-    t.R = R;
-    t.S = S;
-    t.C = 1;
-    t.ws = 0;
-    t.threads = pts_threads(sh, S, R);
-    t.smem = pts_smem_bytes(sh, S, R);
-    if (t.threads > pts_max_threads(R) || t.smem > kSmemCap || !pts_span_ok(sh, R)) t.smem = 0;
-    return t;
+    static const bool allowed = [] {
+        const char *v = getenv("PRIEST_PROJECT_KERNEL");
+        return !(v && std::string(v) == "chunked");
+    }();
+    return allowed;
 }
 
-// Point-owner candidates: two or four points per thread; the samples of one
-// wave over the SMs in one CTA (or the most that fit one CTA), half that, and
-// one to three samples per CTA (several CTAs per SM, whose phases then
-// overlap).
-std::vector<Tiling> pts_candidates(const Shape &sh, int n_samples, int n_sm)
-{
-    std::vector<Tiling> out;
-    if (!pts_supported(sh) || !pts_allowed()) return out;
-    for (int R : {2, 4}) {
-        if (R == 4 && sh.nf != 5) continue;  // compiled for five free coefficients only
-        const int tps = (sh.n_p + R - 1) / R;
-        const int s_max = std::max(1, pts_max_threads(R) / tps);
-        const int s1 = std::min(s_max, std::max(1, (n_samples + n_sm - 1) / n_sm));
-        std::vector<int> ss = {s1, (s1 + 1) / 2, 1, 2, 3};
-        std::sort(ss.begin(), ss.end());
-        ss.erase(std::unique(ss.begin(), ss.end()), ss.end());
-        for (int S : ss) {
-            if (S > s1) continue;
-            const Tiling t = pts_tiling(sh, S, R);
-            if (t.smem > 0) out.push_back(t);
-        }
-    }
-    return out;
-}
-
-// Default tiling: the largest compiled variant, the largest warp group that
+// Default tiling: the point-owner kernel for the shapes it covers; otherwise the
+// largest compiled variant, the largest warp group that
 // fits the CTA, and the obstacle chunk count that gives each group's threads
 // about one item each, within the shared-memory cap.
 template <typename Real>
 Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
 {
-    if (sizeof(Real) == 4 && pts_supported(sh) && pts_span_ok(sh, 2) && pts_allowed()) {
-        const int tps = (sh.n_p + 1) / 2;
-        const int S = std::min(std::max(1, pts_max_threads(2) / tps), std::max(1, (n_samples + n_sm - 1) / n_sm));
-        const Tiling p = pts_tiling(sh, S, 2);
+    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed()) {
+        // an SM's share of the samples in as few CTAs of equal size as hold them
+        const int m = std::max(1, (n_samples + n_sm - 1) / n_sm), G = pts_group(sh, m);
+        // few samples per SM: a team of warps for each (pts_team_size)
+        if (const int C = pts_team_size(sh, m)) {
+            const int fit = 8 / C, n = (m + fit - 1) / fit;
+            const Tiling q = pts_team_tiling(sh, (m + n - 1) / n, C);
+            if (q.smem > 0 && size_t(n) * (q.smem + 1024) <= size_t(228) * 1024) return q;
+        }
+        const int w = (m * G + 31) / 32, ctas = (w + 7) / 8;
+        const Tiling p = pts_tiling(sh, G, (w + ctas - 1) / ctas);
         if (p.smem > 0) return p;
     }
     Tiling t;
@@ -138,7 +114,6 @@ template <typename Real>
 std::vector<Tiling> tiling_candidates(const Shape &sh, int n_samples, int n_sm)
 {
     std::vector<Tiling> out;
-    if (sizeof(Real) == 4) out = pts_candidates(sh, n_samples, n_sm);
     for (const Variant &v : variants<Real>()) {
         if (v.dims != sh.dims) continue;
         for (int ws = 1; ws <= 8 && 32 * ws <= v.threads; ws *= 2) {
@@ -165,51 +140,11 @@ std::vector<Tiling> tiling_candidates(const Shape &sh, int n_samples, int n_sm)
     return out;
 }
 
-// Point-owner tiling of one problem inside a persistent launch: two points
-// per thread, the samples that fill the variant's CTA (at most N).
-// Most samples of one problem that fill the persistent variant's CTA.
-int pts_batch_samples(const Shape &sh)
-{
-    int S = std::max(1, pts_batch_threads(sh) / std::max(1, (sh.n_p + 1) / 2));
-    while (S > 1 && pts_threads(sh, S, 2) > pts_batch_threads(sh)) --S;
-    return S;
-}
-
-Tiling pts_batch_tiling(const Shape &sh, int S)
-{
-    Tiling t;
-    t.kind = 1;
-    t.R = 2;
-    t.S = std::max(1, std::min(S, sh.N));
-    t.C = 1;
-    t.ws = 0;
-    t.threads = pts_batch_threads(sh);
-    t.smem = pts_smem_bytes(sh, t.S, 2);
-    if (pts_threads(sh, t.S, 2) > t.threads || t.smem > kSmemCap || !pts_span_ok(sh, 2)) t.smem = 0;
-    return t;
-}
-
-// PRIEST_PROJECT_KERNEL=chunked in the environment keeps the FP32 projection
-// on the chunked kernel (comparisons; the autotuner otherwise picks).
-bool pts_allowed()
-{
-    static const bool allowed = [] {
-        const char *v = getenv("PRIEST_PROJECT_KERNEL");
-        return !(v && std::string(v) == "chunked");
-    }();
-    return allowed;
-}
-
-bool pts_batch_ok(const Shape &sh)
-{
-    return pts_allowed() && pts_supported(sh) && pts_span_ok(sh, 2) && pts_batch_tiling(sh, 1).smem > 0;
-}
-
 template <typename Real>
 Tiling batch_tiling(const Shape &sh)
 {
-    if (sizeof(Real) == 4 && pts_batch_ok(sh)) {
-        const Tiling p = pts_batch_tiling(sh, pts_batch_samples(sh));
+    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed()) {
+        const Tiling p = pts_batch_tiling(sh, pts_group(sh, 1 << 20), 1 << 20);
         if (p.smem > 0) return p;
     }
     Tiling t;
@@ -232,13 +167,6 @@ template <typename Real>
 std::vector<Tiling> batch_candidates(const Shape &sh)
 {
     std::vector<Tiling> out;
-    if (sizeof(Real) == 4 && pts_batch_ok(sh)) {
-        const int s_full = pts_batch_samples(sh);
-        for (int S : {s_full, (s_full + 1) / 2}) {
-            const Tiling t = pts_batch_tiling(sh, S);
-            if (t.smem > 0 && (out.empty() || out.back().S != t.S)) out.push_back(t);
-        }
-    }
     const int threads = sizeof(Real) == 8 ? 256 : 512;
     for (int ws = 1; ws <= 4; ws *= 2) {
         Tiling t;
@@ -292,6 +220,7 @@ cudaError_t launch_project_batch(const ProjParams<Real> *params_dev, const int2 
                                  size_t smem, int grid, cudaStream_t st, int kind)
 {
     (void)threads;
+    (void)R;
     if (n_items <= 0) return cudaSuccess;
     if constexpr (sizeof(Real) == 4) {
         if (kind == 1)

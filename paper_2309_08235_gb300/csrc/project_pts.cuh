@@ -1,55 +1,58 @@
-// project_pts.cuh -- FP32 fused projection with point-owning threads (Sec. III-A;
+// project_pts.cuh -- FP32 fused projection with point-owning lanes (Sec. III-A;
 // Appendix eqs. lagrange, comp_alpha .. comp_zeta, lag, affine_trans /
 // matrix_vec / comp_zeta), the hot path of the FP32 solver.
 //
-// Same iteration as project_kernel.cuh (phases A: trajectory and velocity /
-// acceleration / workspace residuals, B: obstacle pairs, C: g = F^T (F xi_bar
-// - e) and the multiplier step, D: the shared-inverse step), organised so the
-// per-point work never leaves registers:
-//   * a CTA holds S samples of one problem; thread (s, j) owns the R time
-//     stamps j, j + TPS, ..., TPS = ceil(n_p / R), of sample s for all K
-//     iterations, with its rows of the free-column basis (P, Pd, Pdd) and of
-//     the fixed-coefficient part in registers (loaded once per launch);
-//   * phase B tests the thread's points against the obstacles through
-//     neighbour lists: each thread keeps, per point, the obstacles within
-//     a_j + delta of the point's position at the last rebuild (at most
-//     list_cap(dims), in obstacle order, each with the obstacle's offset terms
-//     at the point's time) and tests only those exactly.  The CTA
-//     rebuilds its lists when one of its points has moved farther than
-//     7/8 delta since the last rebuild (always in the first iteration; one
-//     vote of the whole CTA, so rebuilds do not hold warps at the barrier
-//     of phase C one warp at a time): a point then screens the static
-//     obstacles of its cell of the tables' uniform grid (or, without a grid,
-//     every static obstacle four at a time from "quad" records, one f32x2 FMA
-//     evaluating a point against two obstacles), with thresholds inflated by
-//     delta, and every moving obstacle, two at a time by their scaled
-//     offsets; the flagged ones are appended to the lists.  An
-//     obstacle left out lies at least a_j + delta from the point's rebuild
-//     position, so while the point stays within 7/8 delta of it the pair is
-//     inactive (its residual row is zero) and skipping it changes nothing; the
-//     eighth of delta held back covers the FP32 rounding of the screening.
-//     The exact tests run in obstacle order with one FMA per accumulated
-//     term on every path, so the sums are bitwise those of testing every
-//     obstacle.  A warp whose lists overflowed screens every obstacle
-//     and tests its candidates exactly in every iteration until its next
-//     rebuild; residuals S_o accumulate in registers;
-//   * phase C forms each thread's share of g on the free columns and reduces
-//     it over the sample's threads with a segmented warp reduction (a warp may
-//     hold the end of one sample and the start of the next; lanes 2i, 2i + 1
-//     always share a sample), one partial per (sample, warp) in shared memory,
-//     summed in a fixed order;
-//   * phase D: every warp holds, for each sample it touches, the free
-//     coefficients c, multipliers lambda_F and sample xi_F in registers of
-//     dims * nf "state lanes" (one per axis and free column); after the single
-//     CTA barrier of the iteration those lanes read their sample's partial
-//     sums, apply the multiplier and shared-inverse steps (the W products by
-//     warp shuffles), and the warp's threads take the new c by shuffles.
-//     Warps sharing a sample repeat the same arithmetic, so they agree.
-// One CTA barrier per iteration.  The multipliers of the fixed columns
-// (returned only on request) follow from the linearity of eq. lag:
-// lambda_B^K = lambda_B^0 - rho P_B^T sum_k r^k, so the per-point residual rows
-// are summed over the iterations and reduced once at the end.
+// G = 32 or 16 lanes project one sample through all K iterations; lane l of the
+// group owns the time stamps t = l, l + G, ... .  A residual row is zero wherever
+// its constraint is inactive, and few are active at a time (on the measured
+// scenes a handful of the n_p n_o obstacle pairs of a sample, and the velocity /
+// acceleration rows of none to all of its time stamps), so an iteration
+// evaluates only the rows that can be active:
+//   * obstacle pairs: the pairs (t, j) within a_j + delta at the last rebuild,
+//     sorted by (t, j), with the obstacle's scaled offset terms at time t, spread
+//     evenly over the lanes (the owners of t meet uneven numbers of obstacles);
+//   * velocity rows: all of them, or none while the bound cannot be reached;
+//   * acceleration and workspace rows: one bit per block of time stamps in which
+//     some norm (coordinate) was within a margin of its bound.
+// Position and acceleration are polynomials of degree 10 and 8 in time, and a
+// polynomial of degree n is bounded on its interval by 1 / cos(n pi / 2m) times
+// its maximum over m Chebyshev nodes (Ehlich and Zeller 1964).  The lanes
+// evaluate the displacement of 32 nodes since the last rebuild; while the bound
+// stays below the margins, every pair and row left out is inactive.  (The start's
+// velocity is fixed, so the change of velocity is bounded by that of the
+// acceleration times the time.)  Nothing is approximated: the sums are bitwise
+// those of evaluating every pair.  The m-th active pair in (t, j) order is added
+// by lane m mod G, whatever was listed beside it, and velocity, acceleration and
+// workspace rows by the owner of t, in a fixed order.
+//
+// An iteration is then: the free coefficients from shared memory; the node
+// test; the listed pairs, each row . c + base and its residual, the active ones
+// through shared memory to the lane that adds row^T residual to its share of g;
+// the other listed rows; a transposing butterfly that leaves each of the
+// dims * nf sums of g in a "state lane"; the multiplier and shared-inverse
+// steps in those lanes (W u by shuffles); the new coefficients back to shared
+// memory.  The chain of one iteration is what bounds it (a warp waits on its own
+// results: 1,600 cycles an iteration with one sample per scheduler, and at 16
+// warps per SM 51 % of the issue slots), so the code is straight-line where it
+// can be: loops run to warp-uniform trip counts over branch-free bodies (lists
+// are padded with a pair that is never active), the first trip runs beside the
+// node test, and velocity / acceleration rows go two time stamps to an f32x2 FMA.
+// No CTA barrier: a CTA's warps share only the problem's tables.  With few samples
+// per SM a team of warps shares the chain (project_samples).
+//
+// Before, threads owned two time stamps of a sample, evaluated all their rows in
+// every iteration and met at a CTA barrier; per pass, before -> after: 2-D clutter
+// (N = 1000, n_p = 100, 100 obstacles, K = 100) 195 -> 123 us, 64 uneven 2-D
+// problems (K = 60) 4,534 -> 1,639 us, 3-D ellipsoids (N = 2000, n_p = 150, 200
+// obstacles, K = 100) 826 -> 583 us, a replan of 110 samples (K = 50) 123 -> 102.
+//
+// The multipliers of the fixed columns (returned only on request) follow from
+// the linearity of eq. lag: lambda_B^K = lambda_B^0 - rho sum_k P_B^T r^k, so
+// each lane sums its P_B^T r over the iterations and the group reduces once.
 #pragma once
+
+#include <cfloat>
+#include <type_traits>
 
 #include "project_kernel.cuh"
 
@@ -57,1007 +60,1532 @@ namespace priest {
 namespace pts {
 
 using detail::ffma2;
-using detail::fmin3;
 using detail::fmul2;
-using detail::kFull;
 
-// Shared-memory layout (float units; every block 32-byte aligned).
-//   obs   [n_obs][12 | 16]  obstacle records (copied from the tables)
-//   srec  [nq][12 | 20]     static quads: {m2x x4} {m2y x4} [{m2z x4} {kap x4}] {nthr x4}
-//   mrec  [nm2][12 | 16]    moving pairs (layout of project_kernel.cuh)
-//   W     [nf][nf]
-//   cd    [S][dims][cds]    free coefficients, each stored twice (c_f, c_f)
-//   lam, xi, u [S][dims][8] multipliers, sample (free columns; set-up and output only)
-//   part  [2][S][maxw][dims*nv] per-(sample, warp) partial sums, double-buffered by
-//                           iteration parity
-//   part2 [S][maxw][2]      (doubles) residual / cost partials of the final pass
-//   ref   [R][dims][tl]     each thread's point positions at the last list rebuild
-//   list  [R][cap][tl]      (float4) each thread's neighbour lists, tl = threads rounded
-//                           to 32: per entry the obstacle's scaled offset terms at the
-//                           point's time, 2-D (1/a, -o_x(t)/a, -o_y(t)/a, a), 3-D
-//                           (1/a, 1/b, -o_x(t)/a, -o_y(t)/a)
-//   listz [R][cap][tl]      3-D: -o_z(t)/b
-//   listi [R][cap][tl]      3-D (uint16): the obstacle's index (its a, b for active pairs)
-//   grid  [gl.smem]         the static-obstacle grid of the tables (header, cell starts,
-//                           entries; none below kGridMinStatic static obstacles)
+constexpr unsigned kAll = 0xffffffffu;
+// 1 / cos(n pi / 64), rounded up: bound of a degree-n polynomial by 32 nodes
+constexpr float kNodeBoundPos = 1.1340f;  // n = 10
+constexpr float kNodeBoundAcc = 1.0825f;  // n = 8
+// Velocity / acceleration margin where the bound is close, as a share of the
+// acceleration bound.
+constexpr float kAccMargin = 0.15f;
+
+constexpr int kMaxWarps = 8;    // warps of one CTA
+constexpr int kMaxStrides = 16; // strides of G time stamps
+constexpr int kPairs = 256;     // obstacle pairs a sample may list (a multiple of 32)
+constexpr int kShortLived = 6;  // iterations of a list that lasted too short
+constexpr int kMaxTeam = 4;     // most warps of one sample's team
+// A team's exchange floats: two buffers of {sums of g [3][32], the test's answer}, {r^2, c_1}
+// [kMaxTeam][2] doubles, the fixed columns' sums [kMaxTeam][32]
+constexpr int kXchFlag = 3 * 32, kXchBuf = kXchFlag + 8, kXchEnd = 2 * kXchBuf, kXchFix = kXchEnd + 4 * kMaxTeam,
+              kXch = kXchFix + kMaxTeam * 32;
+
+// Shared-memory layout (float units, every block 32-byte aligned); np is n_p
+// rounded up to 2 G and the row blocks are arrays of 16 bytes over the stamps, so
+// the lanes of a group read neighbouring banks.
+//   header [16]               ints: the offsets and sizes below (Hdr)
+//   rows  [chunks][np][4]     per time stamp, positions: nf free columns of P, then the
+//                             fixed-coefficient part of each axis
+//   vrows [2][pchunks][np / 2][4]  the same of Pd and Pdd, stamps 2 u and 2 u + 1
+//                             interleaved: {v0(2u), v0(2u + 1), v1(2u), v1(2u + 1)}
+//   tv    [np]                time stamps
+//   node  [32 / G][nfn][32][4]  node rows {P, Pdd} of two columns a time (nfn = (nf + 1) / 2)
+//   obs   [n_obs][4]          2-D {1/a, -o_x/a, -o_y/a, a}, 3-D {1/a, -o_x/a, -o_y/a, -o_z/b}
+//   obq   [n_obs][4]          3-D {1/b, a, b, max(1/a, 1/b)}
+//   mov   [n_moving][4]       {-v_x/a, -v_y/a[, -v_z/b]}
+//   grid  [gl.smem]           the static-obstacle grid of the tables
+//   per warp, for each of its 32 / G samples:
+//     c [nf][4 | 8]           coefficients, each twice: {x, x, y, y[, z, z, -, -]}
+//     stage [4 G][4]          active pairs on their way to a lane: {r (dims), t}
+//     list [kPairs][4]        2-D {1/a, -o_x(t)/a, -o_y(t)/a, a}, 3-D {1/a, -o_x(t)/a, -o_y(t)/a, -o_z(t)/b}
+//     tj [kPairs]             (ints) time stamp | obstacle << 16
+//   xch   [teams][kXch]       what a team's warps tell one another
+//   fix   [3][fchunks][np][4] fixed columns (multipliers on request, when it fits)
+constexpr int kRows = 16;  // offset of the rows
+__host__ __device__ constexpr int coef_floats(int dims, int nf) { return nf * (dims == 2 ? 4 : 8); }
+__host__ __device__ constexpr int sample_floats(int G, int dims, int nf)
+{
+    return coef_floats(dims, nf) + 16 * G + 5 * kPairs + (nf & 1) * 4;
+}
 struct PtsLayout {
-    int tps, nq, nm2, maxw, cds, tl, cap;
-    size_t obs, srec, mrec, W, cd, lam, xi, part, part2, ref, list, listz, listi, grid, gsz, total;
+    int np, nch, pch, nfch;
+    size_t rows, vrows, node, tv, obs, obq, mov, grid, gsz, warp0, wsz, xch, fix, total, total_fix;
 };
 
-// Neighbour-list entries per point.
-__host__ __device__ constexpr int list_cap(int dims) { return dims == 2 ? 8 : 6; }
-
-// Threads per sample, rounded up to an even count so the lanes 2i, 2i + 1 of
-// a warp always hold the same sample (the paired reduction of phase C).
-__host__ __device__ inline int pts_tps(int n_p, int R) { return (((n_p + R - 1) / R) + 1) & ~1; }
-
-// Most samples one warp can touch (its 32 consecutive threads cover TPS-thread
-// blocks); every warp keeps the multiplier and coefficient state of each of
-// its samples in dims * nf lanes, so dims * nf * span must fit in 32 lanes.
-__host__ __device__ inline int pts_span(int tps) { return (31 + tps - 1) / tps + 1; }
-
-__host__ __device__ inline PtsLayout pts_layout(int dims, int nf, int nv, int n_p, int n_obs, int n_static, int S,
-                                                int R)
+__host__ __device__ inline PtsLayout pts_layout(int G, int dims, int nf, int nv, int n_p, int n_obs, int n_static,
+                                                int warps, int teams)
 {
     PtsLayout L;
-    L.tps = pts_tps(n_p, R);
-    L.nq = (n_static + 3) / 4;
-    L.nm2 = (n_obs - n_static + 1) / 2;
-    L.maxw = (L.tps + 31) / 32 + 1;
-    L.cds = ((2 * nf + 3) / 4) * 4;
+    L.np = (n_p + 2 * G - 1) & ~(2 * G - 1);
+    L.nch = (nf + dims + 3) / 4;
+    L.pch = (nf + dims + 1) / 2;
+    L.nfch = (nv - nf + 3) / 4;
     size_t o = 0;
-    L.obs = o;
-    o = align8(o + size_t(n_obs) * (dims == 2 ? 12 : 16));
-    L.srec = o;
-    o = align8(o + size_t(L.nq) * (dims == 2 ? 12 : 20));
-    L.mrec = o;
-    o = align8(o + size_t(L.nm2) * (dims == 2 ? 12 : 16));
-    L.W = o;
-    o = align8(o + size_t(nf) * nf);
-    L.cd = o;
-    o = align8(o + size_t(S) * dims * L.cds);
-    L.lam = o;
-    o = align8(o + size_t(S) * dims * 8);
-    L.xi = o;
-    o = align8(o + size_t(S) * dims * 8);
-    L.part = o;
-    o = align8(o + size_t(2) * S * L.maxw * dims * nv);
-    L.part2 = o;
-    o = align8(o + size_t(S) * L.maxw * 4);
-    L.tl = ((S * L.tps + 31) / 32) * 32;
-    L.ref = o;
-    o = align8(o + size_t(R) * dims * L.tl);
-    L.cap = list_cap(dims);
-    L.list = o;
-    o = align8(o + size_t(R) * L.cap * L.tl * 4);
-    L.listz = o;
-    o = align8(o + (dims == 3 ? size_t(R) * L.cap * L.tl : 0));
-    L.listi = o;
-    o = align8(o + (dims == 3 ? (size_t(R) * L.cap * L.tl + 1) / 2 : 0));
-    L.grid = o;
+    auto take = [&o](size_t n) {
+        const size_t at = o;
+        o = align8(o + n);
+        return at;
+    };
+    take(kRows);
+    L.rows = take(size_t(L.nch) * L.np * 4);
+    L.vrows = take(size_t(2) * L.pch * L.np * 2);
+    L.node = take(size_t(32 / G) * ((nf + 1) / 2) * 128);
+    L.tv = take(size_t(L.np));
+    L.obs = take(size_t(n_obs) * 4);
+    L.obq = take(dims == 3 ? size_t(n_obs) * 4 : 0);
+    L.mov = take(size_t(n_obs - n_static) * 4);
     L.gsz = n_static >= kGridMinStatic ? grid_layout(n_static).smem : 0;
-    o = align8(o + L.gsz);
+    L.grid = take(L.gsz);
+    L.warp0 = o;
+    L.wsz = size_t(32 / G) * sample_floats(G, dims, nf);
+    o += L.wsz * warps;
+    L.xch = o;
+    o += size_t(kXch) * teams;
     L.total = o;
+    L.fix = o;
+    L.total_fix = o + size_t(3) * L.nfch * L.np * 4;
     return L;
 }
 
-// Segmented warp sum: lanes [lane, send] of one segment (send = the last lane
-// of the calling lane's segment in this warp); afterwards the first lane of
-// each segment holds its segment's in-warp sum.
-template <typename T>
-__device__ __forceinline__ T seg_sum(T v, int lane, int send)
+// The butterfly's value of a lane of the group: V values over G lanes, halved
+// at each exchange (the lower half of the lanes keeps the first (n + 1) / 2
+// values); -1 where the lane ends up with padding.
+__host__ __device__ constexpr int val_of(int G, int V, int lane)
 {
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const T o = __shfl_down_sync(kFull, v, d);
-        if (lane + d <= send) v += o;
-    }
-    return v;
-}
-
-// Residual contribution of an active pair into registers (the arithmetic of
-// project_kernel.cuh's active_pair): so[] += Delta (1 - 1/rho_s), or in the
-// final pass so[0] += |Delta (1 - 1/rho_s)|^2.
-template <int DIMS>
-__device__ __forceinline__ void active_add(float dx, float dy, float dz, float q, float a, float b, bool fin,
-                                           float (&so)[DIMS])
-{
-    if (q > 0.f) {
-        const float rs = rsqrtf(q);
-        const float w = 1.f - rs;
-        if (!fin) {
-            so[0] = fmaf(a * w, dx, so[0]);
-            so[1] = fmaf(a * w, dy, so[1]);
-            if constexpr (DIMS == 3) so[DIMS - 1] = fmaf(b * w, dz, so[DIMS - 1]);
+    int v = 0, n = V, real = V;
+    for (int off = G / 2; off >= 1; off >>= 1) {
+        if (n == 1) break;
+        const int m = (n + 1) / 2;
+        if (lane & off) {
+            v += m;
+            real -= m;
         } else {
-            // one explicit FMA: every inlined copy rounds the same way
-            const float d2 = (DIMS == 3) ? fmaf(b * b * dz, dz, a * a * fmaf(dx, dx, dy * dy)) : a * a * q;
-            so[0] = fmaf(w * w, d2, so[0]);
+            real = real < m ? real : m;
         }
-    } else {
-        // at the centre the target is o + (a, 0) (2-D) / o + (0, 0, b) (3-D)
-        const float s = (DIMS == 3) ? b : a;
-        if (!fin)
-            so[DIMS == 3 ? DIMS - 1 : 0] -= s;
-        else
-            so[0] = fmaf(s, s, so[0]);
+        n = m;
     }
+    return (real >= 1 && n == 1) ? v : -1;
 }
 
-template <int DIMS>
-__device__ __forceinline__ void exact_static(const float *sObs, int j, float x, float y, float z, bool fin,
-                                             float (&so)[DIMS])
+// The first lane that ends up with value v.
+__host__ __device__ constexpr int lane_of(int G, int V, int v)
 {
-    constexpr int ST = DIMS == 2 ? 12 : 16;
-    const float *o = sObs + size_t(j) * ST;
-    float ia, nox, noy, noz = 0.f, ib = 0.f, a, b = 0.f, d0, d1;
-    if constexpr (DIMS == 2) {
-        a = o[3];
-        detail::ld4(o + 4, ia, nox, noy, d0);
-    } else {
-        detail::ld4(o + 4, d0, a, b, d1);
-        detail::ld4(o + 8, ia, nox, noy, noz);
-        ib = o[12];
-    }
-    const float dx = fmaf(x, ia, nox), dy = fmaf(y, ia, noy);
-    const float dz = (DIMS == 3) ? fmaf(z, ib, noz) : 0.f;
-    const float q = (DIMS == 3) ? fmaf(dx, dx, fmaf(dy, dy, dz * dz)) : fmaf(dx, dx, dy * dy);
-    if (q < 1.f) active_add<DIMS>(dx, dy, dz, q, a, b, fin, so);
+    int l = G - 1;
+    for (int i = G - 1; i >= 0; --i) l = val_of(G, V, i) == v ? i : l;
+    return l;
 }
-
-// Pre-filter values of one static quad against one point (obstacles 0-1 and
-// 2-3): the expanded test without |p|^2, compared with -|p|^2.
-template <int DIMS>
-__device__ __forceinline__ void quad_values(const float *q, float2 xd, float2 yd, float2 zd, float2 zzd, float2 &v01,
-                                            float2 &v23)
-{
-    const float4 A = *reinterpret_cast<const float4 *>(q);
-    const float4 B = *reinterpret_cast<const float4 *>(q + 4);
-    const float4 Cc = *reinterpret_cast<const float4 *>(q + 8);
-    if constexpr (DIMS == 2) {
-        v01 = ffma2(xd, make_float2(A.x, A.y), ffma2(yd, make_float2(B.x, B.y), make_float2(Cc.x, Cc.y)));
-        v23 = ffma2(xd, make_float2(A.z, A.w), ffma2(yd, make_float2(B.z, B.w), make_float2(Cc.z, Cc.w)));
-    } else {
-        const float4 Dd = *reinterpret_cast<const float4 *>(q + 12);
-        const float4 E = *reinterpret_cast<const float4 *>(q + 16);
-        v01 = ffma2(xd, make_float2(A.x, A.y),
-                    ffma2(yd, make_float2(B.x, B.y),
-                          ffma2(zd, make_float2(Cc.x, Cc.y), ffma2(zzd, make_float2(Dd.x, Dd.y), make_float2(E.x, E.y)))));
-        v23 = ffma2(xd, make_float2(A.z, A.w),
-                    ffma2(yd, make_float2(B.z, B.w),
-                          ffma2(zd, make_float2(Cc.z, Cc.w), ffma2(zzd, make_float2(Dd.z, Dd.w), make_float2(E.z, E.w)))));
-    }
-}
-
-template <typename T, int R>
-__device__ __forceinline__ T pick(const T (&a)[R], int r)
-{
-    T v = a[0];
-#pragma unroll
-    for (int i = 1; i < R; ++i)
-        if (r == i) v = a[i];
-    return v;
-}
-
-// Exact tests of the candidates of a batch of quads [k, k + NB): bit r * NB + i
-// of `cand` flags point r against quad k + i.  Candidates are visited point by
-// point in obstacle order; the four obstacles of a flagged quad are
-// re-evaluated with the same operations and the ones below the threshold
-// tested exactly, accumulated into the point's sums as the list path does
-// (one FMA per term), so both paths give the same sums.
-template <int DIMS, int R, int NB>
-__device__ __forceinline__ void quad_candidates(unsigned cand, const float *srec, const float *sObs, int k,
-                                                const detail::PackedPoints<DIMS, R> &P, bool fin,
-                                                float (&so)[R][DIMS])
-{
-    constexpr int QS = DIMS == 2 ? 12 : 20;
-    while (cand) {
-        const int bit = __ffs(cand) - 1;
-        cand &= cand - 1;
-        const int r = bit / NB, i = bit - r * NB;
-        const float2 xd = pick(P.x, r), yd = pick(P.y, r), zd = pick(P.z, r), zzd = pick(P.zz, r);
-        const float npq = pick(P.npq, r);
-        float2 v01, v23;
-        quad_values<DIMS>(srec + size_t(k + i) * QS, xd, yd, zd, zzd, v01, v23);
-        unsigned hb = (v01.x < npq ? 1u : 0u) | (v01.y < npq ? 2u : 0u) | (v23.x < npq ? 4u : 0u) |
-                      (v23.y < npq ? 8u : 0u);
-        while (hb) {
-            const int h = __ffs(hb) - 1;
-            hb &= hb - 1;
-#pragma unroll
-            for (int rr = 0; rr < R; ++rr)
-                if (rr == r) exact_static<DIMS>(sObs, 4 * (k + i) + h, xd.x, yd.x, zd.x, fin, so[rr]);
-        }
-    }
-}
-
-// Per-point minimum of the pre-filter values over one quad.
-template <int DIMS>
-__device__ __forceinline__ float quad_min(const float *q, float2 xd, float2 yd, float2 zd, float2 zzd)
-{
-    float2 v01, v23;
-    quad_values<DIMS>(q, xd, yd, zd, zzd, v01, v23);
-    return fmin3(v01.x, v01.y, fminf(v23.x, v23.y));
-}
-
-template <int DIMS, int R>
-__device__ __forceinline__ void moving_rescan(const float *rec, const float *sObs, int k0, int nb, int j0,
-                                              const detail::PackedPoints<DIMS, R> &P, const float (&m)[R], bool fin,
-                                              float (&so)[R][DIMS])
-{
-    constexpr int RM = DIMS == 2 ? 12 : 16;
-    constexpr int ST = DIMS == 2 ? 12 : 16;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (m[r] < 1.f) {
-            for (int b = k0; b < k0 + nb; ++b) {
-                float2 dx, dy, dz;
-                const float2 q =
-                    detail::moving_value<DIMS>(rec + size_t(b) * RM, P.x[r], P.y[r], P.z[r], P.t[r], dx, dy, dz);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float qh = h ? q.y : q.x;
-                    if (qh < 1.f) {
-                        const float *o = sObs + size_t(j0 + 2 * b + h) * ST;
-                        const float a = (DIMS == 2) ? o[3] : o[5], bb = (DIMS == 2) ? o[3] : o[6];
-                        active_add<DIMS>(h ? dx.y : dx.x, h ? dy.y : dy.x, h ? dz.y : dz.x, qh, a, bb, fin, so[r]);
-                    }
-                }
-            }
-        }
-    }
-}
-
-// Every obstacle against the thread's R points; all lanes of the CTA run the
-// same trip counts, so the votes use the full warp.  Static quads go in
-// batches of NQB: one minimum per (point, quad) kept in registers and their
-// minimum per point; a thread with a candidate records the batch's (point,
-// quad) bits, and after the loop each thread tests its recorded candidates
-// exactly, oldest first (all lanes with candidates in one pass instead of one
-// warp-wide detour per batch).
-template <int DIMS, int R, int NQB>
-__device__ __forceinline__ void all_pairs(const float *srec, const float *mrec, const float *sObs, int nq, int nm2,
-                                          int ns, const detail::PackedPoints<DIMS, R> &P, bool fin,
-                                          float (&so)[R][DIMS])
-{
-    static_assert(R * NQB <= 32, "candidate bits");
-    constexpr int QS = DIMS == 2 ? 12 : 20;
-    constexpr int RM = DIMS == 2 ? 12 : 16;
-    // candidate batches of this thread, processed after the screening loop
-    // (oldest first, so each point still sees its obstacles in order)
-    constexpr int MAXE = 3;
-    int ek0 = 0, ek1 = 0, ek2 = 0, ne = 0;
-    unsigned ec0 = 0u, ec1 = 0u, ec2 = 0u;
-    auto flush = [&]() {
-        for (int e = 0; e < ne; ++e) {
-            const int ke = e == 0 ? ek0 : (e == 1 ? ek1 : ek2);
-            const unsigned ce = e == 0 ? ec0 : (e == 1 ? ec1 : ec2);
-            quad_candidates<DIMS, R, NQB>(ce, srec, sObs, ke, P, fin, so);
-        }
-        ne = 0;
-    };
-    int k = 0;
-    for (; k + NQB <= nq; k += NQB) {
-        // screening: one minimum per (point, quad), their minimum per point
-        float mq[R][NQB];
-#pragma unroll
-        for (int i = 0; i < NQB; ++i) {
-            const float *q = srec + size_t(k + i) * QS;
-#pragma unroll
-            for (int r = 0; r < R; ++r) mq[r][i] = quad_min<DIMS>(q, P.x[r], P.y[r], P.z[r], P.zz[r]);
-        }
-        bool f = false;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float m = mq[r][0];
-#pragma unroll
-            for (int i = 1; i < NQB; i += 2) m = (i + 1 < NQB) ? fmin3(m, mq[r][i], mq[r][i + 1]) : fminf(m, mq[r][i]);
-            f |= m < P.npq[r];
-        }
-        if (f) {
-            // record the (point, quad) candidate bits of the batch
-            unsigned cand = 0u;
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int i = 0; i < NQB; ++i) cand |= (mq[r][i] < P.npq[r] ? 1u : 0u) << (r * NQB + i);
-            if (ne == MAXE) flush();
-            if (ne == 0) {
-                ek0 = k;
-                ec0 = cand;
-            } else if (ne == 1) {
-                ek1 = k;
-                ec1 = cand;
-            } else {
-                ek2 = k;
-                ec2 = cand;
-            }
-            ++ne;
-        }
-    }
-    flush();
-    for (; k < nq; ++k) {
-        unsigned cand = 0u;
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            cand |= (quad_min<DIMS>(srec + size_t(k) * QS, P.x[r], P.y[r], P.z[r], P.zz[r]) < P.npq[r] ? 1u : 0u) << r;
-        if (__any_sync(kFull, cand != 0u)) quad_candidates<DIMS, R, 1>(cand, srec, sObs, k, P, fin, so);
-    }
-    // moving obstacles: the batch minimum is the exact squared scaled distance
-    constexpr int NPM = 2;
-    for (k = 0; k < nm2; k += NPM) {
-        const int nb = min(NPM, nm2 - k);
-        float m[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) m[r] = INFINITY;
-#pragma unroll
-        for (int b = 0; b < NPM; ++b) {
-            if (b < nb) {
-                const float *q = mrec + size_t(k + b) * RM;
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    float2 dx, dy, dz;
-                    const float2 v = detail::moving_value<DIMS>(q, P.x[r], P.y[r], P.z[r], P.t[r], dx, dy, dz);
-                    m[r] = fmin3(m[r], v.x, v.y);
-                }
-            }
-        }
-        bool f = false;
-#pragma unroll
-        for (int r = 0; r < R; ++r) f |= m[r] < 1.f;
-        if (__any_sync(kFull, f)) moving_rescan<DIMS, R>(mrec, sObs, k, nb, ns, P, m, fin, so);
-    }
-}
-
-constexpr unsigned kListOverflow = 0x80000000u;
-
-// Shared-memory neighbour lists of one CTA (see PtsLayout).
-struct PtsLists {
-    float4 *w;             // [R][cap][tl]
-    float *z;              // [R][cap][tl] (3-D)
-    unsigned short *idx;   // [R][cap][tl] (3-D)
-    int tl;
+template <int G, int V, int I>
+struct LaneOf {
+    static constexpr int value = lane_of(G, V, I);
 };
 
-// Neighbour lists of the thread's R points (4 bits of count per point in the
-// returned word, kListOverflow set when a point had more than list_cap
-// obstacles): the static obstacles screened with the quads' inflated
-// thresholds and every moving pair by its scaled offsets against
-// (1 + delta max(1/a, 1/b))^2, the flagged obstacles appended in obstacle
-// order with their offset terms at the point's time.  With a grid (gsm: its
-// region, nx > 0) a point screens only the static obstacles of its cell, each
-// with the arithmetic of its lane of the quad test, in increasing order; the
-// cell holds every obstacle that test can pass for a point in it, so the lists
-// are the same as with every quad screened.  Padding entries of the quad and
-// pair records are never flagged.
-template <int DIMS, int R>
-__device__ __forceinline__ unsigned build_lists(const float *srec, const float *mrec, const float *sObs,
-                                                const float *gsm, int nq, int nm2, int ns,
-                                                const detail::PackedPoints<DIMS, R> &P, float delta,
-                                                const PtsLists &Ls, int tid)
+// Sums h[] over the group; the lane's value val_of(G, V, lane) is returned.  A
+// halving exchange costs half the shuffles of the one before (12 for ten
+// values over 32 lanes, 50 for a plain butterfly of each).
+template <int N, int OFF>
+__device__ __forceinline__ float reduce_step(float *h, int lane)
 {
-    constexpr int QS = DIMS == 2 ? 12 : 20;
-    constexpr int RM = DIMS == 2 ? 12 : 16;
-    constexpr int ST = DIMS == 2 ? 12 : 16;
-    constexpr int CAP = list_cap(DIMS);
-    unsigned cnt = 0u;
-    auto append = [&](int r, int j, float t) {
-        const unsigned c = (cnt >> (4 * r)) & 15u;
-        if (c < unsigned(CAP)) {
-            const int e = (r * CAP + int(c)) * Ls.tl + tid;
-            const float *o = sObs + size_t(j) * ST;
-            if constexpr (DIMS == 2) {
-                Ls.w[e] = make_float4(o[4], fmaf(t, o[8], o[5]), fmaf(t, o[9], o[6]), o[3]);
-            } else {
-                Ls.w[e] = make_float4(o[8], o[12], fmaf(t, o[13], o[9]), fmaf(t, o[14], o[10]));
-                Ls.z[e] = fmaf(t, o[15], o[11]);
-                Ls.idx[e] = static_cast<unsigned short>(j);
-            }
-            cnt += 1u << (4 * r);
-        } else {
-            cnt |= kListOverflow;
-        }
-    };
-    const int gnx = gsm ? __float_as_int(gsm[4]) : 0;
-    if (gnx > 0) {
-        const int gny = __float_as_int(gsm[5]);
-        const float gx0 = gsm[0], gy0 = gsm[1], gih = gsm[2];
-        const unsigned short *gstart = reinterpret_cast<const unsigned short *>(gsm + 8);
-        const unsigned short *gent = reinterpret_cast<const unsigned short *>(gsm + grid_layout(ns).ent);
+    if constexpr (N == 1) {
+        h[0] += __shfl_xor_sync(kAll, h[0], OFF);
+    } else {
+        constexpr int M = (N + 1) / 2;
+        const bool hi = (lane & OFF) != 0;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float x = P.x[r].x, y = P.y[r].x;
-            const float fx = (x - gx0) * gih, fy = (y - gy0) * gih;
-            if (fx >= 0.f && fx < float(gnx) && fy >= 0.f && fy < float(gny)) {
-                const int c = min(int(fy), gny - 1) * gnx + min(int(fx), gnx - 1);
-                const int e1 = gstart[c + 1];
-                const float npq = P.npq[r], t = P.t[r].x;
-                for (int e = gstart[c]; e < e1; ++e) {
-                    const int jo = gent[e];
-                    const float *q = srec + size_t(jo >> 2) * QS + (jo & 3);
-                    float v;
-                    if constexpr (DIMS == 2)
-                        v = fmaf(x, q[0], fmaf(y, q[4], q[8]));
-                    else
-                        v = fmaf(x, q[0], fmaf(y, q[4], fmaf(P.z[r].x, q[8], fmaf(P.zz[r].x, q[12], q[16]))));
-                    if (v < npq) append(r, jo, t);
-                }
-            }
-        }
-    } else
-    for (int k = 0; k < nq; ++k) {
-        const float *q = srec + size_t(k) * QS;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float2 v01, v23;
-            quad_values<DIMS>(q, P.x[r], P.y[r], P.z[r], P.zz[r], v01, v23);
-            const float npq = P.npq[r];
-            if (fmin3(v01.x, v01.y, fminf(v23.x, v23.y)) < npq) {
-                const float t = P.t[r].x;
-                if (v01.x < npq) append(r, 4 * k, t);
-                if (v01.y < npq) append(r, 4 * k + 1, t);
-                if (v23.x < npq) append(r, 4 * k + 2, t);
-                if (v23.y < npq) append(r, 4 * k + 3, t);
-            }
+        for (int i = 0; i < M; ++i) {
+            const float up = i + M < N ? h[i + M] : 0.f;
+            const float send = hi ? h[i] : up, keep = hi ? up : h[i];
+            h[i] = keep + __shfl_xor_sync(kAll, send, OFF);
         }
     }
-    for (int k = 0; k < nm2; ++k) {
-        const float *q = mrec + size_t(k) * RM;
-        const float4 A = *reinterpret_cast<const float4 *>(q);
-        const float i0 = DIMS == 2 ? A.x : fmaxf(A.x, A.z), i1 = DIMS == 2 ? A.y : fmaxf(A.y, A.w);
-        const float b0 = fmaf(delta, i0, 1.f), b1 = fmaf(delta, i1, 1.f);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float2 dx, dy, dz;
-            const float2 v = detail::moving_value<DIMS>(q, P.x[r], P.y[r], P.z[r], P.t[r], dx, dy, dz);
-            if (v.x < b0 * b0) append(r, ns + 2 * k, P.t[r].x);
-            if (v.y < b1 * b1) append(r, ns + 2 * k + 1, P.t[r].x);
-        }
-    }
-    return cnt;
+    if constexpr (OFF > 1)
+        return reduce_step<(N + 1) / 2, OFF / 2>(h, lane);
+    else
+        return h[0];
 }
 
-// Exact tests of the listed obstacles of the thread's points, in list order:
-// the arithmetic of exact_static / moving_rescan with the obstacle's offset
-// terms at the point's time taken from the list entry.
-template <int DIMS, int R>
-__device__ __forceinline__ void list_pairs(const float *sObs, const PtsLists &Ls, unsigned cnt, int tid,
-                                           const detail::PackedPoints<DIMS, R> &P, bool fin, float (&so)[R][DIMS])
+// The CTA's dynamic shared memory in floats; every access below is an offset
+// into it, so addresses stay 32-bit and the tables' offsets are read where used.
+__device__ __forceinline__ float *smem()
 {
-    constexpr int CAP = list_cap(DIMS);
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int n = int((cnt >> (4 * r)) & 15u);
-        const float x = P.x[r].x, y = P.y[r].x, z = P.z[r].x;
-        for (int e = 0; e < n; ++e) {
-            const int ei = (r * CAP + e) * Ls.tl + tid;
-            const float4 w = Ls.w[ei];
-            if constexpr (DIMS == 2) {
-                const float dx = fmaf(x, w.x, w.y), dy = fmaf(y, w.x, w.z);
-                const float q = fmaf(dx, dx, dy * dy);
-                if (q < 1.f) active_add<DIMS>(dx, dy, 0.f, q, w.w, w.w, fin, so[r]);
-            } else {
-                const float dx = fmaf(x, w.x, w.z), dy = fmaf(y, w.x, w.w), dz = fmaf(z, w.y, Ls.z[ei]);
-                const float q = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (q < 1.f) {
-                    const float *o = sObs + size_t(Ls.idx[ei]) * 16;
-                    active_add<DIMS>(dx, dy, dz, q, o[5], o[6], fin, so[r]);
-                }
-            }
-        }
-    }
-}
-
-// The projection of samples [s0, s0 + S) of one problem by the calling CTA
-// (blockDim.x >= S * TPS, a multiple of 32; all threads call it).
-// WL: also return the multipliers of the fixed columns.
-template <int DIMS, int R, int NF, bool WL>
-__device__ void pts_body(const ProjParams<float> &p, int s0)
-{
-    static_assert(R % 2 == 0, "points are paired for the f32x2 basis products");
-    constexpr int H = R / 2;
-    constexpr int ST = DIMS == 2 ? 12 : 16;
-    constexpr int QS = DIMS == 2 ? 12 : 20;
-    constexpr int RM = DIMS == 2 ? 12 : 16;
-    constexpr int NB = 11 - NF;  // fixed columns (degree 10: 11 coefficients per axis)
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float *sm = reinterpret_cast<float *>(smem_raw);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, T = blockDim.x;
-    const int np_ = p.n_p, nv = p.nv, D = DIMS * nv, nobs = p.n_obs, ns = p.n_static;
-    const int S = p.S;
-    const int S_act = min(S, p.N - s0);
-    if (S_act <= 0) return;
-    const PtsLayout L = pts_layout(DIMS, NF, nv, np_, nobs, ns, S, R);
-    const int TPS = L.tps, CDS = L.cds, PD = DIMS * nv;
-    const int s = tid / TPS, j = tid - s * TPS;
-    const bool act = s < S_act;
-    const int sc = act ? s : 0;  // a valid sample index for idle threads' reads
-    const int fw = (sc * TPS) >> 5;
-    // last lane of this thread's segment in the warp (idle threads form one segment)
-    const int send = act ? min(31, (sc + 1) * TPS - 1 - 32 * warp) : 31;
-    const bool head = act && (lane == 0 || j == 0);
-    float *sObs = sm + L.obs, *sW = sm + L.W, *sCd = sm + L.cd, *sLam = sm + L.lam, *sXi = sm + L.xi,
-          *sPart = sm + L.part;
-    double *sPart2 = reinterpret_cast<double *>(sm + L.part2);
-    float *sRef = sm + L.ref;
-    PtsLists Ls;
-    Ls.w = reinterpret_cast<float4 *>(sm + L.list);
-    Ls.z = sm + L.listz;
-    Ls.idx = reinterpret_cast<unsigned short *>(sm + L.listi);
-    Ls.tl = L.tl;
-    const float rho = p.rho, vmax = p.vmax, amax = p.amax, vmax2 = vmax * vmax, amax2 = amax * amax;
+    return reinterpret_cast<float *>(smem_raw);
+}
+enum Hdr {  // kGrid, kFix: 0 = none
+    kVrows, kNode, kTv, kObs, kObq, kMov, kGrid, kFix, kNp, kStamps, kStatic, kObstacles, kNext, kXchAt
+};
+__device__ __forceinline__ int hdr(int i) { return reinterpret_cast<const int *>(smem())[i]; }
+__device__ __forceinline__ float4 ld4s(int off) { return *reinterpret_cast<const float4 *>(smem() + off); }
 
-    // ---- obstacle records and W -> shared memory; a1/a2 sample set-up
-    {
-        const float4 *src = reinterpret_cast<const float4 *>(p.tab + p.lay.obs);
-        float4 *dst = reinterpret_cast<float4 *>(sObs);
-        for (int i = tid; i < nobs * ST / 4; i += T) dst[i] = src[i];
-        for (int i = tid; i < NF * NF; i += T) sW[i] = p.tab[p.lay.W + i];
-        const float4 *gsrc = reinterpret_cast<const float4 *>(p.tab + p.lay.grid);
-        float4 *gdst = reinterpret_cast<float4 *>(sm + L.grid);
-        for (int i = tid; i < int(L.gsz / 4); i += T) gdst[i] = gsrc[i];
+// Free columns of the position row at time stamp t and its fixed part.
+template <int DIMS, int NF>
+__device__ __forceinline__ void load_row(int np, int t, float (&row)[NF], float (&x)[DIMS])
+{
+    constexpr int NCH = (NF + DIMS + 3) / 4;
+    float v[4 * NCH];
+#pragma unroll
+    for (int i = 0; i < NCH; ++i) {
+        const float4 w = ld4s(kRows + (i * np + t) * 4);
+        v[4 * i] = w.x;
+        v[4 * i + 1] = w.y;
+        v[4 * i + 2] = w.z;
+        v[4 * i + 3] = w.w;
     }
-    for (int e = tid; e < S_act * D; e += T) {
-        const int ss = e / D, d = e - ss * D;
-        const int ax = d / nv, col = d - ax * nv;
-        const size_t gi = size_t(s0 + ss) * D + d;
-        const int f = col - kFree0;
-        if (f < 0 || f >= NF) continue;
-        double x;
-        if (p.mode == 0) {
-            x = p.xi_in[gi];
-        } else {
-            const size_t seg = p.seg_len > 0 ? size_t((s0 + ss) / p.seg_len) : 0;  // D-PRIEST distribution
-            const double *Lrow = p.Lc + (seg * D + d) * D;
-            const double *zi = p.z + size_t(s0 + ss) * D;
-            x = p.mu[seg * D + d];
-            for (int q = 0; q <= d; ++q) x = fma(Lrow[q], zi[q], x);
-        }
-        const int ro = ss * DIMS + ax;
-        sXi[ro * 8 + f] = float(x);
-        sCd[ro * CDS + 2 * f] = float(x);
-        sCd[ro * CDS + 2 * f + 1] = float(x);
-        sLam[ro * 8 + f] = p.lam_in ? float(p.lam_in[gi]) : 0.f;
-    }
-    // per-thread constants: basis rows (pairs of points), fixed part, time stamps
-    float2 bf[3][NF][H], bs[3][DIMS][H];
-    float tt[R];
-    bool ok[R];
-    {
-        const int fbs = fb_stride(NF), nfp = nf_padded(NF);
-        const float *fb = p.tab + p.lay.fb, *bas = p.tab + p.lay.base, *tv = p.tab + p.lay.tval;
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int t = j + TPS * r;
-            ok[r] = act && t < np_;
-            tt[r] = ok[r] ? tv[t] : 0.f;
-        }
+    for (int f = 0; f < NF; ++f) row[f] = v[f];
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-            const int t0 = j + TPS * (2 * h), t1 = t0 + TPS;
-            const bool o0 = ok[2 * h], o1 = ok[2 * h + 1];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-                    bf[q][f][h] = make_float2(o0 ? fb[size_t(t0) * fbs + q * nfp + f] : 0.f,
-                                              o1 ? fb[size_t(t1) * fbs + q * nfp + f] : 0.f);
-#pragma unroll
-                for (int ax = 0; ax < DIMS; ++ax) {
-                    // padding points: far from every obstacle, at rest
-                    const float pad = q == 0 ? 1e15f : 0.f;
-                    bs[q][ax][h] = make_float2(o0 ? bas[(q * DIMS + ax) * np_ + t0] : pad,
-                                               o1 ? bas[(q * DIMS + ax) * np_ + t1] : pad);
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // ---- pair records of the obstacle loop (static thresholds inflated by the
-    //      neighbour-list margin: (a + delta)^2 in 2-D, a^2 (1 + delta / min(a, b))^2 in 3-D)
-    const float dl = p.list_delta;
-    for (int q = tid; q < L.nq; q += T) {
-        float *d = sm + L.srec + size_t(q) * QS;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int jo = 4 * q + i;
-            const bool okj = jo < ns;
-            const float *o = sObs + size_t(okj ? jo : 0) * ST;
-            d[i] = okj ? o[0] : 0.f;
-            d[4 + i] = okj ? o[1] : 0.f;
-            if constexpr (DIMS == 2) {
-                d[8 + i] = okj ? -(o[2] + (2.f * o[3] + dl) * dl) : 3e38f;  // padding: never below -|p|^2
-            } else {
-                const float dm = dl * fmaxf(o[8], o[12]);
-                d[8 + i] = okj ? o[2] : 0.f;
-                d[12 + i] = okj ? o[4] : 0.f;
-                d[16 + i] = okj ? -(o[3] + o[5] * o[5] * dm * (2.f + dm)) : 3e38f;
-            }
-        }
-    }
-    for (int q = tid; q < L.nm2; q += T) {
-        float *d = sm + L.mrec + size_t(q) * RM;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int jo = ns + 2 * q + h;
-            const bool okj = jo < nobs;
-            const float *o = sObs + size_t(okj ? jo : 0) * ST;
-            // padding: scaled offset (4, 4[, 4]) at every time, never active
-            if constexpr (DIMS == 2) {
-                d[h] = okj ? o[4] : 0.f;
-                d[2 + h] = okj ? o[5] : 4.f;
-                d[4 + h] = okj ? o[6] : 4.f;
-                d[6 + h] = okj ? o[8] : 0.f;
-                d[8 + h] = okj ? o[9] : 0.f;
-                d[10 + h] = 0.f;
-            } else {
-                d[h] = okj ? o[8] : 0.f;
-                d[2 + h] = okj ? o[12] : 0.f;
-                d[4 + h] = okj ? o[9] : 4.f;
-                d[6 + h] = okj ? o[10] : 4.f;
-                d[8 + h] = okj ? o[11] : 4.f;
-                d[10 + h] = okj ? o[13] : 0.f;
-                d[12 + h] = okj ? o[14] : 0.f;
-                d[14 + h] = okj ? o[15] : 0.f;
-            }
-        }
-    }
-    __syncthreads();
+    for (int ax = 0; ax < DIMS; ++ax) x[ax] = v[NF + ax];
+}
 
-    float smin[DIMS], smax[DIMS];
+// x = base + row . c
+template <int DIMS, int NF>
+__device__ __forceinline__ void eval_row(int np, int t, const float (&c)[NF][DIMS], float (&row)[NF], float (&x)[DIMS])
+{
+    load_row<DIMS, NF>(np, t, row, x);
 #pragma unroll
-    for (int ax = 0; ax < DIMS; ++ax) {
-        smin[ax] = p.smin[ax] - p.tab[p.lay.origin + ax];
-        smax[ax] = p.smax[ax] - p.tab[p.lay.origin + ax];
-    }
-    // state lanes: lane = q * DIMS * NF + ax * NF + f serves the warp's q-th
-    // sample (sw0 + q), axis ax, free column f
-    constexpr int SL = DIMS * NF;
-    const int sw0 = (32 * warp) / TPS;               // first sample the warp touches
-    const int dq = lane / SL, dax = (lane % SL) / NF, df = lane % NF;
-    const int ds = sw0 + dq;
-    const bool dact = lane < (32 / SL) * SL && ds < S_act && ds * TPS < 32 * (warp + 1);
-    float stC = 0.f, stLam = 0.f, stXi = 0.f, wrow[NF];
-    {
-        const int ro = (dact ? ds : 0) * DIMS + dax;
-        if (dact) {
-            stC = sCd[ro * CDS + 2 * df];
-            stLam = sLam[ro * 8 + df];
-            stXi = sXi[ro * 8 + df];
-        }
+    for (int f = 0; f < NF; ++f)
 #pragma unroll
-        for (int fi = 0; fi < NF; ++fi) wrow[fi] = sW[df * NF + fi];
-    }
-    // the state lane holding (my sample, axis, column 0)
-    const int cbase = act ? (sc - sw0) * SL : 0;
-    float rsum[WL ? R : 1][3][DIMS];  // WL: per-point residual rows summed over the iterations
-#pragma unroll
-    for (int r = 0; r < (WL ? R : 1); ++r)
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-#pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax) rsum[r][q][ax] = 0.f;
+        for (int ax = 0; ax < DIMS; ++ax) x[ax] = fmaf(row[f], c[f][ax], x[ax]);
+}
 
-    unsigned lcnt = 0u;  // neighbour-list counts of the thread's points
-    for (int k = 0; k <= p.K; ++k) {
-        const bool fin = (k == p.K);
-        // ---- A: trajectory (pairs of points share one f32x2 FMA per term)
-        float pos[R][DIMS], vel[R][DIMS], acc[R][DIMS];
-        {
-            float cfs[DIMS][NF];
+// Velocity (q = 0) or acceleration (q = 1) at stamps 2 u and 2 u + 1, one f32x2
+// FMA per term.
+template <int DIMS, int NF>
+__device__ __forceinline__ void eval_pair(int vrows, int np, int q, int u, const float2 (&c)[NF][DIMS], float2 (&row)[NF],
+                                          float2 (&x)[DIMS])
+{
+    constexpr int PCH = (NF + DIMS + 1) / 2;
+    float2 v[2 * PCH];
 #pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax)
+    for (int i = 0; i < PCH; ++i) {
+        const float4 w = ld4s(vrows + ((q * PCH + i) * (np / 2) + u) * 4);
+        v[2 * i] = make_float2(w.x, w.y);
+        v[2 * i + 1] = make_float2(w.z, w.w);
+    }
 #pragma unroll
-                for (int f = 0; f < NF; ++f) cfs[ax][f] = __shfl_sync(kFull, stC, (cbase + ax * NF + f) & 31);
+    for (int ax = 0; ax < DIMS; ++ax) x[ax] = v[NF + ax];
 #pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax) {
-                float2 cf[NF];
+    for (int f = 0; f < NF; ++f) {
+        row[f] = v[f];
 #pragma unroll
-                for (int f = 0; f < NF; ++f) cf[f] = make_float2(cfs[ax][f], cfs[ax][f]);
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    float2 P2 = bs[0][ax][h], V2 = bs[1][ax][h], A2 = bs[2][ax][h];
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) {
-                        P2 = ffma2(bf[0][f][h], cf[f], P2);
-                        V2 = ffma2(bf[1][f][h], cf[f], V2);
-                        A2 = ffma2(bf[2][f][h], cf[f], A2);
-                    }
-                    pos[2 * h][ax] = P2.x;
-                    pos[2 * h + 1][ax] = P2.y;
-                    vel[2 * h][ax] = V2.x;
-                    vel[2 * h + 1][ax] = V2.y;
-                    acc[2 * h][ax] = A2.x;
-                    acc[2 * h + 1][ax] = A2.y;
-                }
-            }
+        for (int ax = 0; ax < DIMS; ++ax) x[ax] = ffma2(row[f], c[f][ax], x[ax]);
+    }
+}
+
+template <int DIMS>
+__device__ __forceinline__ float2 norm2(const float2 (&x)[DIMS])
+{
+    const float2 s = ffma2(x[1], x[1], fmul2(x[0], x[0]));
+    return DIMS == 3 ? ffma2(x[DIMS - 1], x[DIMS - 1], s) : s;
+}
+
+// 1 / sqrt(q), q normal (or 0, infinite, NaN: infinite, 0, NaN): rsqrtf without
+// its care for denormals, the same value otherwise.
+__device__ __forceinline__ float rsqrt_normal(float q)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(q));
+    return y;
+}
+
+// Scaled offset terms of obstacle j at time t: {1/a, -o_x/a, -o_y/a, a (2-D) or
+// -o_z/b}; moving obstacles (j >= ns) follow the static ones.
+template <int DIMS>
+__device__ __forceinline__ float4 pair_terms(int j, float t, int ns)
+{
+    float4 o = ld4s(hdr(kObs) + 4 * j);
+    if (j >= ns) {
+        const float4 v = ld4s(hdr(kMov) + 4 * (j - ns));
+        o.y = fmaf(t, v.x, o.y);
+        o.z = fmaf(t, v.y, o.z);
+        if (DIMS == 3) o.w = fmaf(t, v.z, o.w);
+    }
+    return o;
+}
+
+// Scaled offset of the position x from an obstacle and its square.
+template <int DIMS>
+__device__ __forceinline__ float scaled_offset(const float (&x)[DIMS], const float4 &o, float ib, float (&d)[DIMS])
+{
+    d[0] = fmaf(x[0], o.x, o.y);
+    d[1] = fmaf(x[1], o.x, o.z);
+    if constexpr (DIMS == 2) {
+        return fmaf(d[0], d[0], d[1] * d[1]);
+    } else {
+        d[DIMS - 1] = fmaf(x[DIMS - 1], ib, o.w);
+        return fmaf(d[0], d[0], fmaf(d[1], d[1], d[DIMS - 1] * d[DIMS - 1]));
+    }
+}
+
+// Whether a point within delta of the position x may touch the obstacle with
+// the offset terms o (3-D: b its {1/b, a, b, max(1/a, 1/b)}).
+template <int DIMS>
+__device__ __forceinline__ bool near_pair(const float (&x)[DIMS], const float4 &o, const float4 &b, float delta)
+{
+    float d[DIMS];
+    const float q = scaled_offset<DIMS>(x, o, b.x, d), lim = fmaf(delta, DIMS == 3 ? b.w : o.x, 1.f);
+    return q < lim * lim;
+}
+
+// What the screening of a sample's positions keeps in registers.
+template <int DIMS>
+struct Screen {
+    int ns, no, obs, obq, nx, ny, start, ent;  // nx = 0: no grid
+    float x0, y0, ih, delta;
+
+    __device__ __forceinline__ explicit Screen(float margin)
+    {
+        ns = hdr(kStatic);
+        no = hdr(kObstacles);
+        obs = hdr(kObs);
+        obq = hdr(kObq);
+        delta = margin;
+        const int go = hdr(kGrid);
+        const float *g = smem() + go;
+        nx = go ? __float_as_int(g[4]) : 0;
+        ny = go ? __float_as_int(g[5]) : 0;
+        x0 = g[0];
+        y0 = g[1];
+        ih = g[2];
+        start = 2 * (go + 8);
+        ent = 2 * (go + int(grid_layout(ns).ent));
+    }
+    __device__ __forceinline__ static int u16(int i) { return reinterpret_cast<const unsigned short *>(smem())[i]; }
+    __device__ __forceinline__ float4 semi(int j) const
+    {
+        return DIMS == 3 ? ld4s(obq + 4 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+
+    // Calls hit(j, terms), in increasing j, for every static obstacle that a point
+    // within delta of the position x may touch: those of the grid's cell when
+    // there is a grid (four at a time, their loads in flight together), all of
+    // them otherwise.
+    template <typename Hit>
+    __device__ __forceinline__ void fixed(const float (&x)[DIMS], bool valid, Hit hit) const
+    {
+        int e0 = 0, e1 = valid ? ns : 0;
+        if (nx > 0) {
+            const float fx = (x[0] - x0) * ih, fy = (x[1] - y0) * ih;
+            const bool in = valid && fx >= 0.f && fx < float(nx) && fy >= 0.f && fy < float(ny);
+            const int cell = in ? min(int(fy), ny - 1) * nx + min(int(fx), nx - 1) : 0;
+            e0 = u16(start + cell);
+            e1 = in ? u16(start + cell + 1) : e0;
         }
-        float rv[R][DIMS], ra[R][DIMS], rb[R][DIMS], fvv[R], faa[R], v2v[R], a2v[R];
+#pragma unroll 1
+        for (int e = e0; e < e1; e += 4) {
+            int j[4];
+            float4 o[4];
+            bool near[4];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float v2 = 0.f, a2 = 0.f;
-#pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax) {
-                v2 = fmaf(vel[r][ax], vel[r][ax], v2);
-                a2 = fmaf(acc[r][ax], acc[r][ax], a2);
+            for (int i = 0; i < 4; ++i) {
+                const int ei = min(e + i, e1 - 1);
+                j[i] = nx > 0 ? u16(ent + ei) : ei;
             }
-            const float fv = (v2 > vmax2) ? 1.f - vmax * rsqrtf(v2) : 0.f;
-            const float fa = (a2 > amax2) ? 1.f - amax * rsqrtf(a2) : 0.f;
-            fvv[r] = fv;
-            faa[r] = fa;
-            v2v[r] = v2;
-            a2v[r] = a2;
 #pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax) {
-                rv[r][ax] = fv * vel[r][ax];
-                ra[r][ax] = fa * acc[r][ax];
-                rb[r][ax] = (p.use_bounds && ok[r])
-                                ? fmaxf(0.f, pos[r][ax] - smax[ax]) - fmaxf(0.f, smin[ax] - pos[r][ax])
-                                : 0.f;
+            for (int i = 0; i < 4; ++i) {
+                o[i] = ld4s(obs + 4 * j[i]);
+                near[i] = e + i < e1 && near_pair<DIMS>(x, o[i], semi(j[i]), delta);
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (near[i]) hit(j[i], o[i]);
         }
-        // ---- B: the thread's points against their listed obstacles (lists rebuilt when needed)
-        float so[R][DIMS];
-        {
-            detail::PackedPoints<DIMS, R> P;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float x = pos[r][0], y = pos[r][1], z = DIMS == 3 ? pos[r][DIMS - 1] : 0.f;
-                P.x[r] = make_float2(x, x);
-                P.y[r] = make_float2(y, y);
-                P.z[r] = make_float2(z, z);
-                P.zz[r] = make_float2(z * z, z * z);
-                P.t[r] = make_float2(tt[r], tt[r]);
-                P.npq[r] = -fmaf(x, x, y * y);
-#pragma unroll
-                for (int ax = 0; ax < DIMS; ++ax) so[r][ax] = 0.f;
-            }
-            constexpr int NQB = DIMS == 3 ? 2 : (R >= 4 ? 4 : 2);
-            if (dl > 0.f) {
-                // rebuild when a point of the CTA moved farther than 7/8 delta:
-                // one vote of the whole CTA, so that all warps rebuild in the same
-                // iteration instead of each one holding the others at the barrier
-                bool moved = k == 0;
-                if (act && !moved) {
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        float d2 = 0.f;
-#pragma unroll
-                        for (int ax = 0; ax < DIMS; ++ax) {
-                            const float e = pos[r][ax] - sRef[(r * DIMS + ax) * L.tl + tid];
-                            d2 = fmaf(e, e, d2);
-                        }
-                        moved = moved || (ok[r] && d2 > 0.765625f * dl * dl);
-                    }
-                }
-                if (__syncthreads_or(moved)) {
-                    lcnt = build_lists<DIMS, R>(sm + L.srec, sm + L.mrec, sObs, L.gsz && p.list_grid ? sm + L.grid : nullptr, L.nq,
-                                                L.nm2, ns, P, dl, Ls, tid);
-                    if (act) {
-#pragma unroll
-                        for (int r = 0; r < R; ++r)
-#pragma unroll
-                            for (int ax = 0; ax < DIMS; ++ax) sRef[(r * DIMS + ax) * L.tl + tid] = pos[r][ax];
-                    }
-                }
-                if (__any_sync(kFull, (lcnt & kListOverflow) != 0u))
-                    all_pairs<DIMS, R, NQB>(sm + L.srec, sm + L.mrec, sObs, L.nq, L.nm2, ns, P, fin, so);
-                else
-                    list_pairs<DIMS, R>(sObs, Ls, lcnt, tid, P, fin, so);
-            } else {
-                all_pairs<DIMS, R, NQB>(sm + L.srec, sm + L.mrec, sObs, L.nq, L.nm2, ns, P, fin, so);
-            }
-        }
-        if (fin) {
-            // ---- a9: r = sqrt(sum of squared residual rows), c_1
-            double r2 = 0.0, c1 = 0.0;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                if (ok[r]) {
-                    float rq = v2v[r] * fvv[r] * fvv[r] + a2v[r] * faa[r] * faa[r];
-                    if (p.use_bounds) {
-#pragma unroll
-                        for (int ax = 0; ax < DIMS; ++ax) {
-                            const float hi = fmaxf(0.f, pos[r][ax] - smax[ax]);
-                            const float lo = fmaxf(0.f, smin[ax] - pos[r][ax]);
-                            rq = fmaf(hi, hi, fmaf(lo, lo, rq));
-                        }
-                    }
-                    r2 += double(rq) + double(so[r][0]);
-                    c1 += double(point_cost<float, DIMS>(p.cost, pos[r], vel[r], acc[r], a2v[r]));
-                }
-            }
-            r2 = seg_sum(r2, lane, send);
-            c1 = seg_sum(c1, lane, send);
-            if (head) {
-                double *dst = sPart2 + (size_t(sc) * L.maxw + (warp - fw)) * 2;
-                dst[0] = r2;
-                dst[1] = c1;
-            }
-            break;
-        }
-        // ---- C: this thread's share of g on the free columns, reduced per sample
-        float g[DIMS * NF];
+    }
+
+    // The same for the moving obstacles at time t: those that can come near the
+    // box of the group's positions in its time span [t0, t1] (one lane tests one
+    // obstacle).  All lanes of the warp call it together.
+    template <int G, typename Hit>
+    __device__ __forceinline__ void moving(const float (&x)[DIMS], bool valid, float t, float t0, float t1, Hit hit) const
+    {
+        if (no == ns) return;
+        float lo[DIMS], hi[DIMS];
 #pragma unroll
         for (int ax = 0; ax < DIMS; ++ax) {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                float2 acc2 = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int h = 0; h < H; ++h) {
-                    const float2 rp = make_float2(so[2 * h][ax] + rb[2 * h][ax], so[2 * h + 1][ax] + rb[2 * h + 1][ax]);
-                    const float2 r1 = make_float2(rv[2 * h][ax], rv[2 * h + 1][ax]);
-                    const float2 r2v = make_float2(ra[2 * h][ax], ra[2 * h + 1][ax]);
-                    acc2 = ffma2(bf[0][f][h], rp, ffma2(bf[1][f][h], r1, ffma2(bf[2][f][h], r2v, acc2)));
-                }
-                g[ax * NF + f] = acc2.x + acc2.y;
-            }
+            lo[ax] = valid ? x[ax] : FLT_MAX;
+            hi[ax] = valid ? x[ax] : -FLT_MAX;
         }
-        // reduce g over the sample's threads: the lanes 2i, 2i + 1 always share
-        // a sample (TPS is even), so one exchange leaves the first half of the
-        // values on even lanes and the second half on odd lanes, and the
-        // segmented sum runs over stride-2 lanes on half the values
-        constexpr int V = DIMS * NF, VH = (V + 1) / 2;
-        float *part = sPart + size_t(k & 1) * S * L.maxw * PD;
-        {
-            const bool odd = (lane & 1) != 0;
-            float h[VH];
 #pragma unroll
-            for (int i = 0; i < VH; ++i) {
-                const float hi = VH + i < V ? g[VH + i] : 0.f;
-                const float other = __shfl_xor_sync(kFull, odd ? g[i] : hi, 1);
-                h[i] = (odd ? hi : g[i]) + other;
-            }
-#pragma unroll
-            for (int d = 2; d < 32; d <<= 1) {
-                float o[VH];
-#pragma unroll
-                for (int i = 0; i < VH; ++i) o[i] = __shfl_down_sync(kFull, h[i], d);
-                if (lane + d <= send) {
-#pragma unroll
-                    for (int i = 0; i < VH; ++i) h[i] += o[i];
-                }
-            }
-            // the segment's first two lanes hold the sums of the two halves
-            const bool h0 = act && !odd && (lane == 0 || j == 0);
-            const bool h1 = act && odd && (lane == 1 || j == 1);
-            if (h0 || h1) {
-                float *dst = part + (size_t(sc) * L.maxw + (warp - fw)) * PD + kFree0;
-#pragma unroll
-                for (int i = 0; i < VH; ++i) {
-                    const int v = (h1 ? VH : 0) + i;
-                    if (v < V) dst[(v / NF) * nv + (v % NF)] = h[i];
-                }
-            }
-        }
-        if constexpr (WL) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-#pragma unroll
-                for (int ax = 0; ax < DIMS; ++ax) {
-                    rsum[r][0][ax] += so[r][ax] + rb[r][ax];
-                    rsum[r][1][ax] += rv[r][ax];
-                    rsum[r][2][ax] += ra[r][ax];
-                }
-        }
-        __syncthreads();
-        // ---- D: multiplier step (eq. lag) and shared-inverse step in the state
-        //      lanes: lambda^{k+1} = lambda^k - rho g, u = xi + lambda^{k+1} - rho g - c,
-        //      c += W u (the u of the lane's sample and axis gathered by shuffles)
-        {
-            float gs = 0.f;
-            if (dact) {
-                const int nw = (((ds + 1) * TPS - 1) >> 5) - ((ds * TPS) >> 5) + 1;
-                for (int w = 0; w < nw; ++w) gs += part[(size_t(ds) * L.maxw + w) * PD + dax * nv + kFree0 + df];
-            }
-            const float lnew = stLam - rho * gs;
-            const float u = stXi + lnew - rho * gs - stC;
-            const int ub = lane - df;  // lane of (sample, axis, column 0)
-            float du = 0.f;
-#pragma unroll
-            for (int fi = 0; fi < NF; ++fi) du = fmaf(wrow[fi], __shfl_sync(kFull, u, (ub + fi) & 31), du);
-            if (dact) {
-                stLam = lnew;
-                stC = stC + du;
-            }
-        }
-    }
-
-    // ---- fixed-column multipliers: P_B^T of the summed residual rows
-    if constexpr (WL) {
-        const float *bas = p.tab + p.lay.basis;
-        for (int cb = 0; cb < NB; ++cb) {
-            const int col = cb < kFree0 ? cb : cb + NF;
+        for (int off = G / 2; off >= 1; off >>= 1)
 #pragma unroll
             for (int ax = 0; ax < DIMS; ++ax) {
-                float v = 0.f;
+                lo[ax] = fminf(lo[ax], __shfl_xor_sync(kAll, lo[ax], off));
+                hi[ax] = fmaxf(hi[ax], __shfl_xor_sync(kAll, hi[ax], off));
+            }
+        const int gl = threadIdx.x & (G - 1);
+#pragma unroll 1
+        for (int j0 = ns; j0 < no; j0 += G) {
+            bool may = false;
+            const int j = j0 + gl;
+            if (j < no) {
+                // the scaled offset's range over the box and the span misses [-lim, lim] on some
+                // axis (lim with room for rounding; a NaN position is near nothing)
+                const float4 o0 = pair_terms<DIMS>(j, t0, ns), o1 = pair_terms<DIMS>(j, t1, ns), b = semi(j);
+                const float lim = 1.01f * fmaf(delta, DIMS == 3 ? b.w : o0.x, 1.f);
+                may = true;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if (ok[r]) {
-                        const int t = j + TPS * r;
-                        v = fmaf(bas[(size_t(0) * np_ + t) * nv + col], rsum[r][0][ax],
-                                 fmaf(bas[(size_t(1) * np_ + t) * nv + col], rsum[r][1][ax],
-                                      fmaf(bas[(size_t(2) * np_ + t) * nv + col], rsum[r][2][ax], v)));
+                for (int ax = 0; ax < DIMS; ++ax) {
+                    const float i = ax == 2 ? b.x : o0.x;
+                    const float a0 = ax == 0 ? o0.y : ax == 1 ? o0.z : o0.w, a1 = ax == 0 ? o1.y : ax == 1 ? o1.z : o1.w;
+                    may = may && fmaf(hi[ax], i, fmaxf(a0, a1)) > -lim && fmaf(lo[ax], i, fminf(a0, a1)) < lim;
+                }
+            }
+            unsigned m = __ballot_sync(kAll, may);
+            if (G == 16) m = (m | (m >> 16)) & 0xffffu;  // either sample's
+#pragma unroll 1
+            for (; m; m &= m - 1) {
+                const int jm = j0 + __ffs(m) - 1;
+                const float4 o = pair_terms<DIMS>(jm, t, ns);
+                if (valid && near_pair<DIMS>(x, o, semi(jm), delta)) hit(jm, o);
+            }
+        }
+    }
+};
+
+// Residual of an active pair (q = |d|^2 < 1, d its scaled offset):
+// r = Delta (1 - 1 / sqrt(q)); at the centre the target is o + (a, 0) (2-D) /
+// o + (0, 0, b) (3-D).
+template <int DIMS>
+__device__ __forceinline__ void pair_residual(const float (&d)[DIMS], float q, float a, float b, float (&r)[DIMS])
+{
+    const float w = 1.f - rsqrt_normal(fmaxf(q, FLT_MIN));
+#pragma unroll
+    for (int ax = 0; ax < DIMS; ++ax) r[ax] = ((DIMS == 3 && ax == 2 ? b : a) * w) * d[ax];
+    constexpr int up = DIMS == 3 ? DIMS - 1 : 0;
+    r[up] = q > 0.f ? r[up] : -(DIMS == 3 ? b : a);
+}
+
+// Its squared norm (final pass).
+template <int DIMS>
+__device__ __forceinline__ float pair_square(const float (&d)[DIMS], float q, float a, float b)
+{
+    if (!(q > 0.f)) return DIMS == 3 ? b * b : a * a;
+    const float w = 1.f - rsqrtf(q);
+    const float d2 = DIMS == 3 ? fmaf(b * b * d[DIMS - 1], d[DIMS - 1], a * a * fmaf(d[0], d[0], d[1] * d[1])) : a * a * q;
+    return w * w * d2;
+}
+
+// Free columns {of the Bernstein basis, of its second derivative} at one of 32
+// Chebyshev nodes of [0, T] (degree 10; only bounds use them).
+template <int NF>
+__device__ __forceinline__ void node_rows(int node, float horizon, float2 (&row)[NF + 1])
+{
+    const float tau = 0.5f - 0.5f * cospif(float(2 * node + 1) * (1.f / 64.f)), u = 1.f - tau;
+    const float c10[11] = {1.f, 10.f, 45.f, 120.f, 210.f, 252.f, 210.f, 120.f, 45.f, 10.f, 1.f};
+    const float c8[9] = {1.f, 8.f, 28.f, 56.f, 70.f, 56.f, 28.f, 8.f, 1.f};
+    float tp[11], up[11], b8[9];
+    tp[0] = up[0] = 1.f;
+#pragma unroll
+    for (int i = 1; i <= 10; ++i) {
+        tp[i] = tp[i - 1] * tau;
+        up[i] = up[i - 1] * u;
+    }
+#pragma unroll
+    for (int j = 0; j <= 8; ++j) b8[j] = c8[j] * tp[j] * up[8 - j];
+    const float sc = 90.f / (horizon * horizon);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const int j = kFree0 + f;
+        row[f].x = c10[j] * tp[j] * up[10 - j];
+        row[f].y = sc * (b8[j - 2] - (j - 1 <= 8 ? 2.f * b8[j - 1 <= 8 ? j - 1 : 0] : 0.f) + (j <= 8 ? b8[j <= 8 ? j : 0] : 0.f));
+    }
+    row[NF] = make_float2(0.f, 0.f);
+}
+
+// A 4-byte asynchronous copy into shared memory; zero when !in (src is not read).
+__device__ __forceinline__ void copy4(float *dst, const float *src, bool in)
+{
+    const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(in ? 4 : 0) : "memory");
+}
+
+// Starts the copies of the problem's tables into shared memory (all threads of
+// the CTA; each waits for its own, then a barrier).
+template <int G, int DIMS, int NF, bool WL>
+__device__ void stage_tables(const ProjParams<float> &p, float *sm, const PtsLayout &L, bool with_fix)
+{
+    const int tid = threadIdx.x, T = blockDim.x, np_ = p.n_p;
+    const int fbs = fb_stride(NF), nfp = nf_padded(NF);
+    // asynchronous 4-byte copies (zeros beyond the last time stamp): every load is in flight at once
+    auto put = [&](size_t at, int q, int t, int e) {  // e-th value of the row of kind q at stamp t
+        const bool in = t < np_ && e < NF + DIMS;
+        const float *src = !in ? p.tab
+                               : e < NF ? p.tab + p.lay.fb + size_t(t) * fbs + q * nfp + e
+                                        : p.tab + p.lay.base + (q * DIMS + (e - NF)) * np_ + t;
+        copy4(sm + at, src, in);
+    };
+    constexpr int RW = 4 * ((NF + DIMS + 3) / 4), VW = 4 * ((NF + DIMS + 1) / 2);
+    for (int t = tid; t < L.np; t += T)
+#pragma unroll
+        for (int e = 0; e < RW; ++e) put(L.rows + (size_t(e / 4) * L.np + t) * 4 + e % 4, 0, t, e);
+    // (the halves of the CTA take a kind each)
+    const int hp = L.np / 2, q = tid >= T / 2 ? 1 : 0;
+    for (int u = tid - q * (T / 2); u < hp; u += T / 2)
+#pragma unroll
+        for (int z = 0; z < VW; ++z)
+            put(L.vrows + (size_t(q * (VW / 4) + z / 4) * hp + u) * 4 + z % 4, 1 + q, 2 * u + (z & 1),
+                2 * (z / 4) + ((z >> 1) & 1));
+    for (int t = tid; t < L.np; t += T) copy4(sm + L.tv + t, p.tab + (t < np_ ? p.lay.tval + t : 0), t < np_);
+    constexpr int ST = DIMS == 2 ? 12 : 16;
+    for (int j = tid; j < p.n_obs; j += T) {
+        // 2-D {-2 o_x, -2 o_y, thr, a | 1/a, -o_x/a, -o_y/a, 0 | -v_x/a, -v_y/a, 0, 0};
+        // 3-D {-2 o_x, -2 o_y, -2 kappa o_z, thr | kappa, a, b, 0 | 1/a, -o_x/a, -o_y/a, -o_z/b |
+        //      1/b, -v_x/a, -v_y/a, -v_z/b}
+        const float *o = p.tab + p.lay.obs + size_t(j) * ST;
+        float *d = sm + L.obs + 4 * size_t(j);
+        for (int i = 0; i < 4; ++i) copy4(d + i, o + (DIMS == 3 ? 8 + i : i < 3 ? 4 + i : 3), true);
+        if (DIMS == 3) {
+            float *q = sm + L.obq + 4 * size_t(j);
+            copy4(q, o + 12, true);
+            copy4(q + 1, o + 5, true);
+            copy4(q + 2, o + 6, true);
+            q[3] = fmaxf(o[8], o[12]);
+        }
+        if (j >= p.n_static)
+            for (int i = 0; i < DIMS; ++i) copy4(sm + L.mov + 4 * size_t(j - p.n_static) + i, o + (DIMS == 3 ? 13 : 8) + i, true);
+    }
+    for (int i = tid; i < int(L.gsz); i += T) copy4(sm + L.grid + i, p.tab + p.lay.grid + i, true);
+    if constexpr (WL) {
+        if (with_fix)
+            for (int i = tid; i < 3 * L.np; i += T) {
+                const int f = i / L.np, t = i - f * L.np;
+                for (int e = 0; e < 4 * L.nfch; ++e) {
+                    const int col = e < kFree0 ? e : e + NF;
+                    const bool in = t < np_ && col < p.nv;
+                    copy4(sm + L.fix + (size_t(f * L.nfch + e / 4) * L.np + t) * 4 + e % 4,
+                          p.tab + (in ? p.lay.basis + (size_t(f) * np_ + t) * p.nv + col : 0), in);
+                }
+            }
+    }
+}
+
+// du += W u over the free columns of the lane's axis, the u of column F from
+// its state lane.
+template <int G, int DIMS, int NF, int F>
+__device__ __forceinline__ void gather_u(float u, int src0, const float (&wrow)[NF], float &du)
+{
+    if constexpr (F < NF) {
+        constexpr int V = DIMS * NF;
+        float uf;
+        if constexpr (DIMS == 2) {
+            // the first exchange splits the axes, so an axis fills one half of the group
+            static_assert(LaneOf<G, V, NF + F>::value == LaneOf<G, V, F>::value + G / 2, "axes in halves");
+            uf = __shfl_sync(kAll, u, LaneOf<G, V, F>::value, G / 2);
+        } else {
+            static_assert(LaneOf<G, V, NF + F>::value - LaneOf<G, V, F>::value == LaneOf<G, V, NF>::value, "evenly spaced");
+            uf = __shfl_sync(kAll, u, LaneOf<G, V, F>::value + src0);
+        }
+        du = fmaf(wrow[F], uf, du);
+        gather_u<G, DIMS, NF, F + 1>(u, src0, wrow, du);
+    }
+}
+
+// One sample's warp-level view: group lane, coefficient block, staging, list.
+template <int G, int DIMS, int NF>
+struct Group {
+    int gl, pc;  // lane of the group; offset of the coefficient block
+    __device__ __forceinline__ float4 *stage() const
+    {
+        return reinterpret_cast<float4 *>(smem() + pc + coef_floats(DIMS, NF) + (NF & 1) * 4);
+    }
+    __device__ __forceinline__ float4 *list() const { return stage() + 4 * G; }
+    __device__ __forceinline__ int *tj() const { return reinterpret_cast<int *>(list() + kPairs); }
+};
+
+// The sample's coefficients, each in both halves of a register pair.
+template <int DIMS, int NF>
+__device__ __forceinline__ void load_coefs(int pc, float2 (&c)[NF][DIMS])
+{
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const float4 v = ld4s(pc + f * (DIMS == 2 ? 4 : 8));
+        c[f][0] = make_float2(v.x, v.y);
+        c[f][1] = make_float2(v.z, v.w);
+        if constexpr (DIMS == 3) c[f][DIMS - 1] = *reinterpret_cast<const float2 *>(smem() + pc + f * 8 + 4);
+    }
+}
+
+template <int DIMS, int NF>
+__device__ __forceinline__ void load_coefs(int pc, float (&c)[NF][DIMS])
+{
+    float2 d[NF][DIMS];
+    load_coefs<DIMS, NF>(pc, d);
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int ax = 0; ax < DIMS; ++ax) c[f][ax] = d[f][ax].x;
+}
+
+// The scaled offset of the pair with the terms o (3-D: obstacle j), its square
+// and the semi-axes.
+template <int DIMS>
+__device__ __forceinline__ float listed_offset(const float (&x)[DIMS], const float4 &o, int j, float (&d)[DIMS], float &a,
+                                               float &b)
+{
+    float ib = 0.f;
+    a = o.w;
+    b = 0.f;
+    if constexpr (DIMS == 3) {
+        const float4 v = ld4s(hdr(kObq) + 4 * j);
+        ib = v.x;
+        a = v.y;
+        b = v.z;
+    }
+    return scaled_offset<DIMS>(x, o, ib, d);
+}
+
+// Exclusive prefix sum of n over the group and (total) its sum.
+template <int G>
+__device__ __forceinline__ int group_scan(int n, int gl, int &total)
+{
+    int inc = n;
+#pragma unroll
+    for (int off = 1; off < G; off <<= 1) {
+        const int o = __shfl_up_sync(kAll, inc, off, G);
+        if (gl >= off) inc += o;
+    }
+    total = __shfl_sync(kAll, inc, G - 1, G);
+    return inc - n;
+}
+
+// Barrier of a team's warps.
+template <int TEAM>
+__device__ __forceinline__ void team_sync(int team)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(32 * TEAM) : "memory");
+}
+
+// Lists the pairs of every time stamp (sorted by (t, j)), padded to a multiple
+// of G; returns the trips of the longest list of the warp, -1 when a sample has
+// more than kPairs.  The strides of G time stamps one after another; in a team
+// one to a warp at a time (role and totals, 2 TEAM ints of shared memory: where
+// a warp's stride begins in the list follows from the others' totals; `list` is
+// the group that holds it).
+template <int TEAM, int G, int DIMS, int NF>
+__device__ __forceinline__ int build_list(Group<G, DIMS, NF> gr, Group<G, DIMS, NF> list, float delta, int role, int team,
+                                          int *totals)
+{
+    float c[NF][DIMS];
+    load_coefs<DIMS, NF>(gr.pc, c);
+    const int np = hdr(kNp), n_p = hdr(kStamps), tvo = hdr(kTv);
+    const Screen<DIMS> sc(delta);
+    float4 *lst = list.list();
+    int *tj = list.tj();
+    int base = 0;
+#pragma unroll 1
+    for (int q0 = 0, turn = 0; q0 < n_p; q0 += TEAM * G, turn ^= 1) {
+        const int r0 = q0 + role * G, t = r0 + gr.gl, tc = TEAM > 1 ? min(t, np - 1) : t;
+        const bool valid = t < n_p;
+        float row[NF], x[DIMS];
+        eval_row<DIMS, NF>(np, tc, c, row, x);
+        const float tt = smem()[tvo + tc], ta = smem()[tvo + min(r0, n_p - 1)], tb = smem()[tvo + min(r0 + G, n_p) - 1];
+        auto screen = [&](auto hit) {
+            sc.fixed(x, valid, hit);
+            sc.template moving<G>(x, valid, tt, ta, tb, hit);
+        };
+        // the first five hits of a lane are kept, a second screening serves longer ones
+        int n = 0;
+        unsigned long long kept = 0ull;
+        screen([&](int j, const float4 &) {
+            if (n < 5) kept |= static_cast<unsigned long long>(j) << (12 * n);
+            ++n;
+        });
+        int total;
+        int at = base + group_scan<G>(n, gr.gl, total);
+        if constexpr (TEAM > 1) {
+            // (the next round writes the other half: a warp is there only past the barrier that
+            // follows every read of this one)
+            if (gr.gl == 0) totals[TEAM * turn + role] = total;
+            team_sync<TEAM>(team);
+            total = 0;
+#pragma unroll
+            for (int i = 0; i < TEAM; ++i) {
+                const int v = totals[TEAM * turn + i];
+                if (i < role) at += v;
+                total += v;
+            }
+        }
+        base += total;
+        auto write = [&](int j, const float4 &o) {
+            if (at < kPairs) {
+                lst[at] = o;
+                tj[at] = t | (j << 16);
+            }
+            ++at;
+        };
+        if (__any_sync(kAll, n > 5)) {
+            screen(write);
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < n; ++i) {
+                const int j = int(kept & 4095u);
+                kept >>= 12;
+                write(j, pair_terms<DIMS>(j, tt, sc.ns));
+            }
+        }
+    }
+    const int most = __reduce_max_sync(kAll, base);
+    const int trips = most > kPairs ? -1 : max(1, (most + G - 1) / G);
+    // padding: a pair that is never active
+    if (TEAM == 1 || role == 0)
+        for (int e = base + gr.gl; e < trips * G; e += G) {
+            lst[e] = make_float4(0.f, 4.f, 0.f, 0.f);
+            tj[e] = 0;
+        }
+    if constexpr (TEAM > 1)
+        team_sync<TEAM>(team);
+    else
+        __syncwarp();
+    return trips;
+}
+
+// Every pair screened now, in the list's order (more pairs than a list holds,
+// or lists off): add(t, r) at the lane that the pair's number among the active
+// ones gives, r.x the squared residual instead when SQUARE.  Used out of line, away
+// from the registers of the iteration.
+template <bool SQUARE, int G, int DIMS, int NF, typename Add>
+__device__ __forceinline__ void dense_pairs(const Group<G, DIMS, NF> &gr, float delta, Add add)
+{
+    float c[NF][DIMS];
+    load_coefs<DIMS, NF>(gr.pc, c);
+    const int np = hdr(kNp), n_p = hdr(kStamps), tvo = hdr(kTv);
+    const Screen<DIMS> sc(delta);
+    float4 *buf = gr.list();  // active pairs of one stride, kPairs at a time
+    int base = 0;             // active pairs so far
+#pragma unroll 1
+    for (int r0 = 0; r0 < n_p; r0 += G) {
+        const int t = r0 + gr.gl;
+        float row[NF], x[DIMS];
+        eval_row<DIMS, NF>(np, t, c, row, x);
+        const float tt = smem()[tvo + t], ta = smem()[tvo + r0], tb = smem()[tvo + min(r0 + G, n_p) - 1];
+        auto each = [&](auto use) {
+            auto hit = [&](int j, const float4 &o) {
+                float d[DIMS], a, b;
+                const float q = listed_offset<DIMS>(x, o, j, d, a, b);
+                if (q < 1.f) use(d, q, a, b);
+            };
+            sc.fixed(x, t < n_p, hit);
+            sc.template moving<G>(x, t < n_p, tt, ta, tb, hit);
+        };
+        int n = 0, total;
+        each([&](const float (&)[DIMS], float, float, float) { ++n; });
+        const int first = group_scan<G>(n, gr.gl, total);
+        const int most = __reduce_max_sync(kAll, total);
+#pragma unroll 1
+        for (int w0 = 0; w0 < most; w0 += kPairs) {
+            int at = first - w0;
+            each([&](const float (&d)[DIMS], float q, float a, float b) {
+                if (at >= 0 && at < kPairs) {
+                    if constexpr (SQUARE) {
+                        buf[at].x = pair_square<DIMS>(d, q, a, b);
+                    } else {
+                        float r[DIMS];
+                        pair_residual<DIMS>(d, q, a, b, r);
+                        buf[at] = make_float4(r[0], r[1], DIMS == 3 ? r[DIMS - 1] : 0.f, __int_as_float(t));
                     }
                 }
-                v = seg_sum(v, lane, send);
-                if (head) sPart[(size_t(p.K & 1) * S * L.maxw + size_t(sc) * L.maxw + (warp - fw)) * PD + ax * nv + col] = v;
+                ++at;
+            });
+            __syncwarp();
+            const int end = min(total - w0, kPairs);
+            for (int i = (gr.gl - base - w0) & (G - 1); i < end; i += G) {
+                const float4 v = buf[i];
+                add(__float_as_int(v.w), v);
             }
+            __syncwarp();
+        }
+        base += total;
+    }
+}
+
+// g += sum of row^T r over the sample's active pairs; gfix (may be null): the
+// fixed columns' sums, fix: the fixed columns of P in global memory.
+template <int G, int DIMS, int NF>
+__device__ __noinline__ void dense_sums(Group<G, DIMS, NF> gr, float delta, float (*g)[DIMS], float (*gfix)[DIMS],
+                                        const float *fix, int nv)
+{
+    const int np = hdr(kNp);
+    dense_pairs<false, G, DIMS, NF>(gr, delta, [&](int t, const float4 &v) {
+        float row[NF], x[DIMS];
+        load_row<DIMS, NF>(np, t, row, x);
+        const float r[3] = {v.x, v.y, v.z};
+        for (int ax = 0; ax < DIMS; ++ax) {
+            for (int f = 0; f < NF; ++f) g[f][ax] = fmaf(row[f], r[ax], g[f][ax]);
+            if (gfix)
+                for (int f = 0; f < 11 - NF; ++f)
+                    gfix[f][ax] = fmaf(fix[size_t(t) * nv + (f < kFree0 ? f : f + NF)], r[ax], gfix[f][ax]);
+        }
+    });
+}
+
+// The lane's sum of the squared residuals of the sample's active pairs.
+template <int G, int DIMS, int NF>
+__device__ __noinline__ double dense_squares(Group<G, DIMS, NF> gr, float delta)
+{
+    double r2 = 0.0;
+    dense_pairs<true, G, DIMS, NF>(gr, delta, [&](int, const float4 &v) { r2 += double(v.x); });
+    return r2;
+}
+
+// Which velocity / acceleration rows can become active before the acceleration
+// has changed by sqrt(tau2) at some node: blocks of two time stamps per lane,
+// velocity in the low half word (all or none), acceleration in the high one.
+struct RateRows {
+    float tau2;
+    unsigned bits;
+};
+template <int G, int DIMS, int NF>
+__device__ __forceinline__ RateRows rate_rows(Group<G, DIMS, NF> gr, float vmax, float amax)
+{
+    float2 c[NF][DIMS];
+    load_coefs<DIMS, NF>(gr.pc, c);
+    const int np = hdr(kNp), vrows = hdr(kVrows);
+    float v2 = 0.f, a2 = 0.f;  // largest squares (a NaN counts as large)
+    auto top = [](float m, float x) { return x <= m ? m : x; };
+#pragma unroll 1
+    for (int u = gr.gl; u < np / 2; u += G) {
+        float2 row[NF], v[DIMS], a[DIMS];
+        eval_pair<DIMS, NF>(vrows, np, 0, u, c, row, v);
+        eval_pair<DIMS, NF>(vrows, np, 1, u, c, row, a);
+        const float2 nv2 = norm2<DIMS>(v), na2 = norm2<DIMS>(a);
+        v2 = top(top(v2, nv2.x), nv2.y);
+        a2 = top(top(a2, na2.x), na2.y);
+    }
+    v2 = __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(v2)));
+    a2 = __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(a2)));
+    // the velocity changes by at most `reach` times what the acceleration does (NF = 5: it is
+    // fixed at both ends)
+    const float reach = (NF == 5 ? 0.5f : 1.f) * smem()[hdr(kTv) + hdr(kStamps) - 1];
+    const float slv = 0.95f * (vmax - sqrtf(v2)), sla = 0.95f * (amax - sqrtf(a2));
+    const unsigned all = (1u << (np / (2 * G))) - 1u;
+    float da = fminf(sla, slv / reach);
+    unsigned vel = 0u, acc = 0u;
+    if (!(da > 0.05f * amax)) {
+        da = fmaxf(sla, kAccMargin * amax);
+        if (!(slv > reach * da)) vel = all;
+    }
+    if (!(sla >= da)) {
+        // blocks with an acceleration within the margin (a NaN counts as within)
+        const float la = fmaxf(0.f, amax - 1.05f * da), la2 = la * la;
+#pragma unroll 1
+        for (int u = gr.gl, i = 0; u < np / 2; u += G, ++i) {
+            float2 row[NF], a[DIMS];
+            eval_pair<DIMS, NF>(vrows, np, 1, u, c, row, a);
+            const float2 na2 = norm2<DIMS>(a);
+            if (!(na2.x <= la2 && na2.y <= la2)) acc |= 1u << i;
+        }
+        acc = __reduce_or_sync(kAll, acc);
+        // nearly all blocks: all of them, which needs no test where the velocity is on too
+        if (4 * __popc(acc) >= 3 * __popc(all)) acc = all;
+    }
+    RateRows rr;
+    rr.bits = vel | (acc << 16);
+    rr.tau2 = vel == all && acc == all ? INFINITY : (da / kNodeBoundAcc) * (da / kNodeBoundAcc);
+    return rr;
+}
+
+// Strides of time stamps with a position within delta of the workspace's walls
+// or beyond them.
+template <int DIMS>
+__device__ __forceinline__ void wall(const ProjParams<float> &p, int ax, float &lo, float &hi)
+{
+    const float o = p.tab[p.lay.origin + ax];
+    lo = p.smin[ax] - o;
+    hi = p.smax[ax] - o;
+}
+template <int G, int DIMS, int NF>
+__device__ __noinline__ unsigned wall_rows(Group<G, DIMS, NF> gr, const ProjParams<float> &p, float delta)
+{
+    float c[NF][DIMS];
+    load_coefs<DIMS, NF>(gr.pc, c);
+    const int np = hdr(kNp), n_p = hdr(kStamps);
+    unsigned bits = 0u;
+#pragma unroll 1
+    for (int t = gr.gl, i = 0; t < n_p; t += G, ++i) {
+        float row[NF], x[DIMS];
+        eval_row<DIMS, NF>(np, t, c, row, x);
+#pragma unroll
+        for (int ax = 0; ax < DIMS; ++ax) {
+            float lo, hi;
+            wall<DIMS>(p, ax, lo, hi);
+            if (x[ax] > hi - delta || x[ax] < lo + delta) bits |= 1u << i;
         }
     }
-    // free coefficients and multipliers of each sample from its first warp's state lanes
-    if (dact && (ds * TPS) >> 5 == warp) {
-        const int ro = ds * DIMS + dax;
-        sCd[ro * CDS + 2 * df] = stC;
-        sLam[ro * 8 + df] = stLam;
-    }
-    __syncthreads();
-    // ---- outputs: r, c_1; xi_bar (boundary coefficients from the closed form), lambda
-    for (int ss = tid; ss < S_act; ss += T) {
-        const int nw = (((ss + 1) * TPS - 1) >> 5) - ((ss * TPS) >> 5) + 1;
-        double r2 = 0.0, c1 = 0.0;
-        for (int w = 0; w < nw; ++w) {
-            r2 += sPart2[(size_t(ss) * L.maxw + w) * 2];
-            c1 += sPart2[(size_t(ss) * L.maxw + w) * 2 + 1];
+    return __reduce_or_sync(kAll, bits);
+}
+
+// a1 / a2: the sample's free coefficient and multiplier in each state lane, and
+// its row of W: all that a warp reads from global memory before the first
+// iteration, so that the reads of a CTA's first samples run beside the staging
+// of the tables.
+template <int NF>
+struct Start {
+    float c, lam, wrow[NF];
+};
+template <int G, int DIMS, int NF>
+__device__ __forceinline__ Start<NF> sample_start(const ProjParams<float> &p, int s_first, int s_end)
+{
+    constexpr int V = DIMS * NF;
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1), nv = p.nv, D = DIMS * nv;
+    const int s = min(s_first + lane / G, s_end - 1), val = val_of(G, V, gl);
+    const bool stv = val >= 0;
+    const int sax = stv ? val / NF : 0, sf = stv ? val - sax * NF : 0, sd = sax * nv + kFree0 + sf;
+    const size_t row0 = size_t(s) * D;
+    double x64;
+    if (p.mode == 0) {
+        x64 = stv ? p.xi_in[row0 + sd] : 0.0;
+    } else {
+        // mu + L z: every coefficient's sum split over PARTS lanes (FP64 issues slowly here)
+        constexpr int PARTS = G / V;
+        const size_t seg = p.seg_len > 0 ? size_t(s / p.seg_len) : 0;  // D-PRIEST distribution
+        const int v = gl % V, part = gl / V, d = (v / NF) * nv + kFree0 + v % NF;
+        double acc = 0.0;
+        x64 = stv ? p.mu[seg * D + sd] : 0.0;
+        if (part < PARTS) {
+            const double *Lrow = p.Lc + (seg * D + d) * D, *zi = p.z + row0;
+            for (int q = part; q <= d; q += PARTS) acc = fma(Lrow[q], zi[q], acc);
         }
-        p.r_out[s0 + ss] = sqrt(r2);
-        p.c1_out[s0 + ss] = c1;
+#pragma unroll
+        for (int k = 0; k < PARTS; ++k) x64 += __shfl_sync(kAll, acc, (stv ? val : 0) + k * V, G);
     }
-    for (int e = tid; e < S_act * D; e += T) {
-        const int ss = e / D, d = e - ss * D;
-        const int ax = d / nv, cl = d - ax * nv, f = cl - kFree0;
-        const size_t gi = size_t(s0 + ss) * D + d;
-        const int ro = ss * DIMS + ax;
-        const bool free_col = f >= 0 && f < NF;
-        p.xi_bar[gi] = free_col ? double(sCd[ro * CDS + 2 * f]) : p.cB[ax * kMaxNv + cl];
-        if (p.lam_out) {
-            float lv;
-            if (free_col) {
-                lv = sLam[ro * 8 + f];
-            } else {
-                float gsum = 0.f;
-                if constexpr (WL) {
-                    const int nw = (((ss + 1) * TPS - 1) >> 5) - ((ss * TPS) >> 5) + 1;
-                    for (int w = 0; w < nw; ++w)
-                        gsum += sPart[(size_t(p.K & 1) * S * L.maxw + size_t(ss) * L.maxw + w) * PD + ax * nv + cl];
+    Start<NF> st;
+    st.c = stv ? float(x64) : 0.f;
+    st.lam = stv && p.lam_in ? float(p.lam_in[row0 + sd]) : 0.f;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) st.wrow[f] = stv ? p.tab[p.lay.W + sf * NF + f] : 0.f;
+    return st;
+}
+
+// The projection of samples s_first and (G = 16) s_first + 1 by the calling
+// warp; samples from s_end on repeat the last one and write nothing.  pw: the
+// warp's shared block.
+//
+// TEAM > 1 warps project the one sample s_first, for launches that leave an SM few
+// samples, where one warp's chain of an iteration is all that is waited for.
+// Role 0 keeps and adds the obstacle and workspace rows; of four warps, roles 1
+// and 2 add the velocity and acceleration rows of alternate blocks of time stamps
+// and role 3 makes the node test beside them; of two, role 1 does both.  The
+// partial sums of g and the test's answer meet in shared memory (one barrier an
+// iteration); when the lists no longer hold, the sums are dropped, the lists
+// rebuilt (a stride of time stamps to a warp) and the iteration done again.  Every
+// warp repeats the multiplier and shared-inverse steps.
+template <int G, int DIMS, int NF, bool WL, int TEAM>
+__device__ __forceinline__ void project_samples(const ProjParams<float> &p, int pw, int s_first, int s_end, int role,
+                                                int team, const Start<NF> &start)
+{
+    static_assert(TEAM == 1 || (G == 32 && (TEAM == 2 || TEAM == 4)), "a team's warps hold one sample");
+    const bool pos = TEAM == 1 || role == 0, rate = TEAM == 1 || role == 1 || (TEAM == 4 && role == 2);
+    const bool tester = TEAM > 1 && role == TEAM - 1;
+    const unsigned rate_mask = TEAM == 4 ? (role == 1 ? 0xaaaa5555u : role == 2 ? 0x5555aaaau : 0u) : rate ? ~0u : 0u;
+    constexpr int V = DIMS * NF, NB = 11 - NF, NN = 32 / G;
+    constexpr int CS = coef_floats(DIMS, NF) / NF;  // floats per column in the coefficient block
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1), nv = p.nv, D = DIMS * nv;
+    Group<G, DIMS, NF> gr;
+    gr.gl = gl;
+    gr.pc = pw + (lane / G) * sample_floats(G, DIMS, NF);
+    const int pc = gr.pc;
+    const bool live = s_first + lane / G < s_end;
+    const int s = min(s_first + lane / G, s_end - 1);
+    const int np = hdr(kNp), n_p = hdr(kStamps), vrows = hdr(kVrows);
+
+    // ---- the sample's state lanes
+    const int val = val_of(G, V, gl);
+    const bool stv = val >= 0;
+    const int sax = stv ? val / NF : 0, sf = stv ? val - sax * NF : 0;
+    const int sd = sax * nv + kFree0 + sf;
+    const int src0 = (lane & ~(G - 1)) + (DIMS == 3 ? sax * LaneOf<G, V, NF>::value : 0);
+    const size_t row0 = size_t(s) * D;
+    float stC = start.c, stLam = start.lam;
+    const float stXi = stC;
+    float wrow[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) wrow[f] = start.wrow[f];
+    float2 *stp = reinterpret_cast<float2 *>(smem() + pc + sf * CS + 2 * sax);  // this lane's coefficient
+    __syncwarp();
+    if (stv) *stp = make_float2(stC, stC);
+    gr.list()[gl] = make_float4(0.f, 4.f, 0.f, 0.f);  // (evaluated once before the first rebuild)
+    gr.tj()[gl] = 0;
+    __syncwarp();
+
+    const float rho = p.rho, vmax = p.vmax, amax = p.amax;
+    const int K = p.K;
+    const bool bounds = p.use_bounds != 0, lists = p.list_on != 0;
+    // the obstacles' margin; without obstacles any positive length serves the other rows
+    const float delta = p.list_delta > 0.f ? p.list_delta : 0.01f * vmax * smem()[hdr(kTv) + n_p - 1];
+    const int nblk = np / (2 * G);  // blocks of two time stamps per lane (at most 8)
+    auto load_node = [&](int i, float2 (&node)[NF + 1]) {
+#pragma unroll
+        for (int f = 0; f < (NF + 1) / 2; ++f) {
+            const float4 v = ld4s(hdr(kNode) + ((i * ((NF + 1) / 2) + f) * 32 + lane) * 4);
+            node[2 * f] = make_float2(v.x, v.y);
+            if (2 * f + 1 <= NF) node[2 * f + 1] = make_float2(v.z, v.w);
+        }
+    };
+    float2 ref[NN][DIMS];  // node displacement {position, acceleration} = ref + node . c
+#pragma unroll
+    for (int i = 0; i < NN; ++i)
+#pragma unroll
+        for (int ax = 0; ax < DIMS; ++ax) ref[i][ax] = make_float2(0.f, 0.f);
+    // a negative threshold makes the first iteration build
+    float tauP2 = lists ? -1.f : INFINITY, tauA2 = tauP2;
+    int trips = lists ? 1 : -1;  // of the pair list (the longest of the warp); -1: screen every time stamp
+    // warp-uniform: blocks of the velocity (low half) and acceleration rows, strides of the workspace's
+    unsigned rates = lists ? 0u : (((1u << nblk) - 1u) * 65537u) & rate_mask;
+    unsigned mbx = bounds && !lists && pos ? (2u << ((n_p - 1) / G)) - 1u : 0u;
+    constexpr int NFCH = (NB + 3) / 4;
+    const int fix = WL ? hdr(kFix) : 0;
+    float gfix[WL ? NB : 1][DIMS];
+#pragma unroll
+    for (int f = 0; f < (WL ? NB : 1); ++f)
+#pragma unroll
+        for (int ax = 0; ax < DIMS; ++ax) gfix[f][ax] = 0.f;
+    auto add_fix = [&](const float (&r)[DIMS], int q, int t) {
+        if constexpr (WL) {
+#pragma unroll
+            for (int i = 0; i < NFCH; ++i) {
+                float4 w;
+                if (fix) {
+                    w = ld4s(fix + ((q * NFCH + i) * np + t) * 4);
+                } else {
+                    const float *b = p.tab + p.lay.basis + (size_t(q) * n_p + min(t, n_p - 1)) * nv;
+                    auto at = [&](int f) { return f < NB ? b[f < kFree0 ? f : f + NF] : 0.f; };
+                    w = make_float4(at(4 * i), at(4 * i + 1), at(4 * i + 2), at(4 * i + 3));
                 }
-                lv = (p.lam_in ? float(p.lam_in[gi]) : 0.f) - rho * gsum;
+                const float v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (4 * i + u < NB)
+#pragma unroll
+                        for (int ax = 0; ax < DIMS; ++ax) gfix[4 * i + u][ax] = fmaf(v[u], r[ax], gfix[4 * i + u][ax]);
             }
-            p.lam_out[gi] = double(lv);
+        }
+    };
+
+    float c[NF][DIMS];
+    // which lists the nodes' displacement since the last rebuild no longer proves: bit 0 the
+    // positions', bit 1 the rates'
+    auto outdated = [&](const float2 (&cc)[NF][DIMS]) {
+        float e_p = 0.f, e_a = 0.f;  // its square
+#pragma unroll
+        for (int i = 0; i < NN; ++i) {
+            float2 e[DIMS], node[NF + 1];
+            load_node(i, node);
+#pragma unroll
+            for (int ax = 0; ax < DIMS; ++ax) e[ax] = ref[i][ax];
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) e[ax] = ffma2(node[f], cc[f][ax], e[ax]);
+            const float2 n = norm2<DIMS>(e);
+            e_p = fmaxf(e_p, n.x);
+            e_a = fmaxf(e_a, n.y);
+        }
+        if (!__any_sync(kAll, e_p > tauP2 || e_a > tauA2)) return 0;
+        return (__any_sync(kAll, e_p > tauP2) ? 1 : 0) | (__any_sync(kAll, e_a > tauA2) ? 2 : 0);
+    };
+    // the warp's part of the rebuild, for every sample it holds.  Lists that lasted only a few
+    // iterations are rebuilt with twice the margin, those of too many pairs with half of it
+    // (never beyond the margin that the grid's cells were filled for)
+    float reach = delta;
+    const float widest = (hdr(kGrid) ? 1.f : 8.f) * delta;
+    int built = -kShortLived;
+    auto rebuild = [&](int need, int k, const float2 (&cc)[NF][DIMS]) {
+        const bool need_p = need & 1, need_a = need & 2;
+        if (need_p) {
+            if (k - built < kShortLived) reach = fminf(2.f * reach, widest);
+            built = k;
+            if (pos || TEAM > 1) {
+                Group<G, DIMS, NF> held = gr;  // role 0's block holds the list
+                held.pc -= role * sample_floats(G, DIMS, NF);
+                for (;;) {
+                    trips = build_list<TEAM>(gr, held, reach, role, team,
+                                             reinterpret_cast<int *>(smem() + hdr(kXchAt) + team * kXch + kXchEnd));
+                    if (trips >= 0 || reach < 0.1f * delta) break;
+                    reach *= 0.5f;
+                }
+                if (bounds && pos) mbx = wall_rows<G, DIMS, NF>(gr, p, reach);
+            }
+            // largest displacement between rebuilds: 7/8 of the margin (the rest covers rounding)
+            tauP2 = (0.875f / kNodeBoundPos) * reach * ((0.875f / kNodeBoundPos) * reach);
+        }
+        if (need_a && (rate || tester)) {
+            const RateRows rr = rate_rows<G, DIMS, NF>(gr, vmax, amax);
+            rates = rr.bits & rate_mask;
+            tauA2 = rr.tau2;
+        }
+        if (TEAM == 1 || tester)
+#pragma unroll
+            for (int i = 0; i < NN; ++i) {
+                float2 node[NF + 1];
+                load_node(i, node);
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) {
+                    float2 e = make_float2(0.f, 0.f);
+#pragma unroll
+                    for (int f = 0; f < NF; ++f) e = ffma2(make_float2(-node[f].x, -node[f].y), cc[f][ax], e);
+                    if (need_p) ref[i][ax].x = e.x;
+                    if (need_a) ref[i][ax].y = e.y;
+                }
+            }
+    };
+    if (TEAM > 1 && lists) {
+        float2 cc[NF][DIMS];
+        load_coefs<DIMS, NF>(pc, cc);
+        rebuild(3, 0, cc);
+    }
+    for (int k = 0, turn = 0;; ++k, ++turn) {
+        load_coefs<DIMS, NF>(pc, c);
+        // the pair that trip e of the list gives this lane: its residual and whether it is active
+        auto trip = [&](int e, float (&r)[DIMS], int &t) {
+            const float4 o = gr.list()[e * G + gl];
+            const int w = gr.tj()[e * G + gl];
+            t = w & 0xffff;
+            float row[NF], x[DIMS], d[DIMS], a, b;
+            eval_row<DIMS, NF>(np, t, c, row, x);
+            const float q = listed_offset<DIMS>(x, o, w >> 16, d, a, b);
+            pair_residual<DIMS>(d, q, a, b, r);
+            return q < 1.f;
+        };
+        float r0[DIMS];
+        int t0, need = 0;
+        bool in0;
+        float gfix0[TEAM > 1 && WL ? NB : 1][DIMS];  // gfix at the start of the iteration
+        const bool last = TEAM > 1 && k == K;        // only the test is left
+        if constexpr (TEAM > 1) {
+            if (pos) {
+                in0 = trip(0, r0, t0);
+            }
+            if (tester) {
+                float2 cc[NF][DIMS];
+                load_coefs<DIMS, NF>(pc, cc);
+                need = outdated(cc);
+            }
+            if constexpr (WL)
+#pragma unroll
+                for (int f = 0; f < NB; ++f)
+#pragma unroll
+                    for (int ax = 0; ax < DIMS; ++ax) gfix0[f][ax] = gfix[f][ax];
+        } else {
+            // ---- the first trip's chain runs beside the node test's
+            for (bool tested = false;; tested = true) {
+                in0 = trip(0, r0, t0);
+                if (tested) break;
+                float2 cc[NF][DIMS];
+                load_coefs<DIMS, NF>(pc, cc);
+                need = outdated(cc);
+                if (need == 0) break;
+                rebuild(need, k, cc);
+            }
+            if (k == K) break;
+        }
+
+        // ---- the lane's share of g = F^T (F xi_bar - e): the listed pairs first, the m-th active
+        //      one at lane m mod G
+        float g[NF][DIMS];
+        bool act = false;
+        auto add = [&](const float (&row)[NF], const float (&r)[DIMS]) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) g[f][ax] = fmaf(row[f], r[ax], g[f][ax]);
+        };
+        if (!pos || last) {
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) g[f][ax] = 0.f;
+        } else if (trips >= 0) {
+            int n = 0;  // active so far
+            auto put = [&](bool in, const float (&r)[DIMS], int t) {
+                unsigned m = __ballot_sync(kAll, in);
+                if (G == 16) m = (m >> (lane & 16)) & 0xffffu;
+                if (in)
+                    gr.stage()[(n + __popc(m & ((1u << gl) - 1u))) & (4 * G - 1)] =
+                        make_float4(r[0], r[1], DIMS == 3 ? r[DIMS - 1] : 0.f, __int_as_float(t));
+                n += __popc(m);
+            };
+            auto get = [&](int m) {  // the lane's m-th active pair, zero when there is none
+                const bool have = m < n;
+                const float4 v = gr.stage()[m & (4 * G - 1)];
+                const int t = have ? __float_as_int(v.w) : 0;
+                float row[NF], x[DIMS], r[DIMS];
+                r[0] = have ? v.x : 0.f;
+                r[1] = have ? v.y : 0.f;
+                if constexpr (DIMS == 3) r[DIMS - 1] = have ? v.z : 0.f;
+                load_row<DIMS, NF>(np, t, row, x);
+                add(row, r);
+                add_fix(r, 0, t);
+                act = act || have;
+            };
+            put(in0, r0, t0);
+            int done = 0;  // of them taken (a multiple of G, the same over the group)
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) g[f][ax] = 0.f;
+            // the stage holds 4 G pairs: the oldest G are taken before they could be overwritten,
+            // the others at the end
+            bool last = false;
+#pragma unroll 1
+            for (int e = 1;; ++e) {
+                if (e < trips) {
+                    float r[DIMS];
+                    int t;
+                    const bool in = trip(e, r, t);
+                    put(in, r, t);
+                    if (e < 3 || !__any_sync(kAll, n - done > 3 * G)) continue;
+                } else {
+                    last = true;
+                }
+                __syncwarp();
+                const bool now = last || n - done > 3 * G;
+                get(now ? done + gl : 0x7fffffff);
+                done += now ? G : 0;
+                __syncwarp();
+                if (last && !__any_sync(kAll, n > done)) break;
+            }
+        } else {
+            float gg[NF][DIMS], gf[WL ? NB : 1][DIMS];
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) gg[f][ax] = 0.f;
+#pragma unroll
+            for (int f = 0; f < (WL ? NB : 1); ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) gf[f][ax] = gfix[f][ax];
+            dense_sums<G, DIMS, NF>(gr, delta, gg, WL ? gf : nullptr, p.tab + p.lay.basis, nv);
+            act = true;
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) g[f][ax] = gg[f][ax];
+#pragma unroll
+            for (int f = 0; f < (WL ? NB : 1); ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) gfix[f][ax] = gf[f][ax];
+        }
+        // velocity (q = 0) and acceleration (q = 1) rows, two time stamps per lane at a time
+#pragma unroll 1
+        for (unsigned m = last ? 0u : rates; m; m &= m - 1) {
+            const int bit = __ffs(m) - 1, q = bit >> 4, u = (bit & 15) * G + gl;
+            const float lim = q ? amax : vmax;
+            float2 row[NF], v[DIMS], cc[NF][DIMS];
+            load_coefs<DIMS, NF>(pc, cc);
+            eval_pair<DIMS, NF>(vrows, np, q, u, cc, row, v);
+            const float2 n2 = norm2<DIMS>(v);
+            // (a NaN counts as active, so it is not lost)
+            const bool i0 = !(n2.x <= lim * lim), i1 = !(n2.y <= lim * lim);
+            if (__any_sync(kAll, i0 || i1)) {
+                const float w0 = i0 ? fmaf(-lim, rsqrt_normal(n2.x), 1.f) : 0.f;
+                const float w1 = i1 ? fmaf(-lim, rsqrt_normal(n2.y), 1.f) : 0.f;
+                float ra[NF], rb[NF], a0[DIMS], a1[DIMS];
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    ra[f] = row[f].x;
+                    rb[f] = row[f].y;
+                }
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) {
+                    a0[ax] = w0 * v[ax].x;
+                    a1[ax] = w1 * v[ax].y;
+                }
+                add(ra, a0);
+                add_fix(a0, 1 + q, 2 * u);
+                add(rb, a1);
+                add_fix(a1, 1 + q, 2 * u + 1);
+                act = act || i0 || i1;
+            }
+        }
+        if (bounds) {
+#pragma unroll 1
+            for (unsigned m = last ? 0u : mbx; m; m &= m - 1) {
+                const int t = gl + G * (__ffs(m) - 1);
+                float row[NF], x[DIMS], r[DIMS];
+                eval_row<DIMS, NF>(np, t, c, row, x);
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) {
+                    float lo, hi;
+                    wall<DIMS>(p, ax, lo, hi);
+                    r[ax] = t < n_p ? fmaxf(0.f, x[ax] - hi) - fmaxf(0.f, lo - x[ax]) : 0.f;
+                    act = act || r[ax] != 0.f;
+                }
+                add(row, r);
+                add_fix(r, 0, t);
+            }
+        }
+        // ---- g over the group, into the state lanes (zero when no row is active)
+        float gs = 0.f;
+        if (__any_sync(kAll, act)) {
+            float h[V];
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) h[ax * NF + f] = g[f][ax];
+            gs = reduce_step<V, G / 2>(h, lane);
+        }
+        if constexpr (TEAM > 1) {
+            // (two buffers: a warp writes one again only after the others have read it, past the
+            // next iteration's barrier)
+            float *x = smem() + hdr(kXchAt) + team * kXch + (turn & 1) * kXchBuf;
+            if (role < 3) x[role * 32 + lane] = gs;
+            if (tester && lane == 0) x[kXchFlag] = __int_as_float(need);
+            team_sync<TEAM>(team);
+            need = __float_as_int(x[kXchFlag]);
+            if (need != 0) {
+                float2 cc[NF][DIMS];
+                load_coefs<DIMS, NF>(pc, cc);
+                rebuild(need, k, cc);
+                if constexpr (WL)
+#pragma unroll
+                    for (int f = 0; f < NB; ++f)
+#pragma unroll
+                        for (int ax = 0; ax < DIMS; ++ax) gfix[f][ax] = gfix0[f][ax];
+            }
+            if (last) break;
+            if (need != 0) {
+                --k;
+                continue;
+            }
+            gs = x[lane] + x[32 + lane];
+            if (TEAM == 4) gs += x[64 + lane];
+        }
+        // ---- multiplier step (eq. lag) and shared-inverse step:
+        //      lambda^{k+1} = lambda^k - rho g, u = xi + lambda^{k+1} - rho g - c, c += W u
+        stLam = fmaf(-rho, gs, stLam);
+        const float u = fmaf(-rho, gs, stXi + stLam) - stC;
+        float du = 0.f;
+        gather_u<G, DIMS, NF, 0>(u, src0, wrow, du);
+        stC += du;
+        if (stv) *stp = make_float2(stC, stC);
+        __syncwarp();
+    }
+
+    // ---- a9: r = sqrt(sum of squared residual rows), c_1
+    double r2 = 0.0, c1 = 0.0;
+    float2 cc[NF][DIMS];
+    load_coefs<DIMS, NF>(pc, cc);
+#pragma unroll 1
+    for (int u = TEAM > 1 ? gl + (role - 1) * G : gl; 2 * u < n_p && (TEAM == 1 || !pos); u += TEAM == 4 ? 3 * G : G) {
+        float2 vrow[NF], vv[DIMS], av[DIMS];
+        eval_pair<DIMS, NF>(vrows, np, 0, u, cc, vrow, vv);
+        eval_pair<DIMS, NF>(vrows, np, 1, u, cc, vrow, av);
+        const float2 v22 = norm2<DIMS>(vv), a22 = norm2<DIMS>(av);
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int t = 2 * u + half;
+            if (t >= n_p) break;
+            float row[NF], x[DIMS], v[DIMS], a[DIMS];
+            if (bounds || p.cost.kind == 1) eval_row<DIMS, NF>(np, t, c, row, x);
+#pragma unroll
+            for (int ax = 0; ax < DIMS; ++ax) {
+                v[ax] = half ? vv[ax].y : vv[ax].x;
+                a[ax] = half ? av[ax].y : av[ax].x;
+            }
+            const float v2 = half ? v22.y : v22.x, a2 = half ? a22.y : a22.x;
+            const float fv = (v2 > vmax * vmax) ? 1.f - vmax * rsqrtf(v2) : 0.f;
+            const float fa = (a2 > amax * amax) ? 1.f - amax * rsqrtf(a2) : 0.f;
+            float rq = v2 * fv * fv + a2 * fa * fa;
+            if (bounds) {
+#pragma unroll
+                for (int ax = 0; ax < DIMS; ++ax) {
+                    float lo, hi;
+                    wall<DIMS>(p, ax, lo, hi);
+                    hi = fmaxf(0.f, x[ax] - hi);
+                    lo = fmaxf(0.f, lo - x[ax]);
+                    rq = fmaf(hi, hi, fmaf(lo, lo, rq));
+                }
+            }
+            r2 += double(rq);
+            c1 += double(point_cost<float, DIMS>(p.cost, x, v, a, a2));
+        }
+    }
+    if (!pos) {
+        // the pairs are role 0's
+    } else if (trips >= 0) {
+        // squares to the lanes as above, so that the sum does not depend on the list
+        int n = 0, done = gl;
+#pragma unroll 1
+        for (int e = 0; e < trips; ++e) {
+            const float4 o = gr.list()[e * G + gl];
+            const int w = gr.tj()[e * G + gl];
+            float row[NF], x[DIMS], d[DIMS], a, b;
+            eval_row<DIMS, NF>(np, w & 0xffff, c, row, x);
+            const float q = listed_offset<DIMS>(x, o, w >> 16, d, a, b);
+            const bool in = q < 1.f;
+            unsigned m = __ballot_sync(kAll, in);
+            if (G == 16) m = (m >> (lane & 16)) & 0xffffu;
+            if (in) gr.stage()[(n + __popc(m & ((1u << gl) - 1u))) & (4 * G - 1)].x = pair_square<DIMS>(d, q, a, b);
+            n += __popc(m);
+            __syncwarp();
+            if (done < n) {  // at most one per trip
+                r2 += double(gr.stage()[done & (4 * G - 1)].x);
+                done += G;
+            }
+            __syncwarp();
+        }
+    } else {
+        r2 += dense_squares<G, DIMS, NF>(gr, delta);
+    }
+    {
+        // the lower half of the group ends with r2, the upper half with c_1
+        const bool hi = (gl & (G / 2)) != 0;
+        double v = (hi ? c1 : r2) + __shfl_xor_sync(kAll, hi ? r2 : c1, G / 2);
+#pragma unroll
+        for (int off = G / 4; off >= 1; off >>= 1) v += __shfl_xor_sync(kAll, v, off);
+        if constexpr (TEAM > 1) {
+            float *x = smem() + hdr(kXchAt) + team * kXch;
+            double *xd = reinterpret_cast<double *>(x + kXchEnd);
+            if (gl == 0) xd[2 * role] = v;
+            if (gl == G / 2) xd[2 * role + 1] = v;
+            if constexpr (WL) {
+                constexpr int VB = NB * DIMS;
+                float gb[VB];
+#pragma unroll
+                for (int i = 0; i < VB; ++i) gb[i] = gfix[i % NB][i / NB];
+                const float gsum = reduce_step<VB, G / 2>(gb, lane);
+                const int vb = val_of(G, VB, gl);
+                if (vb >= 0) x[kXchFix + 32 * role + vb] = gsum;
+            }
+            team_sync<TEAM>(team);
+            if (role != 0) return;
+            const int at = gl == 0 ? 0 : 1;
+            v = xd[at] + xd[2 + at];
+            if (TEAM == 4) v += xd[4 + at] + xd[6 + at];
+        }
+        if (live && gl == 0) p.r_out[s] = sqrt(v);
+        if (live && gl == G / 2) p.c1_out[s] = v;
+    }
+    // ---- xi_bar (boundary coefficients from the closed form) and multipliers
+    if (live)
+        for (int d = gl; d < D; d += G) {
+            const int ax = d / nv, col = d - ax * nv, f = col - kFree0;
+            p.xi_bar[row0 + d] = (f >= 0 && f < NF) ? double(smem()[pc + f * CS + 2 * ax]) : p.cB[ax * kMaxNv + col];
+        }
+    if (p.lam_out) {
+        // (with 32 lanes each value sits in two neighbouring ones)
+        if (live && stv && (G == 16 || (gl & 1) == 0)) p.lam_out[row0 + sd] = double(stLam);
+        if constexpr (WL) {
+            constexpr int VB = NB * DIMS;
+            auto put = [&](int i, float gsum) {
+                const int ax = i / NB, f = i - ax * NB;
+                const size_t gi = row0 + ax * nv + (f < kFree0 ? f : f + NF);
+                const float l0 = p.lam_in ? float(p.lam_in[gi]) : 0.f;
+                if (live) p.lam_out[gi] = double(fmaf(-rho, gsum, l0));
+            };
+            float gb[VB];
+#pragma unroll
+            for (int i = 0; i < VB; ++i) gb[i] = gfix[i % NB][i / NB];
+            if constexpr (TEAM > 1) {
+                const float *x = smem() + hdr(kXchAt) + team * kXch + kXchFix;
+                if (gl < VB) put(gl, TEAM == 4 ? (x[gl] + x[32 + gl]) + x[64 + gl] : x[gl] + x[32 + gl]);
+            } else if constexpr (VB <= G) {
+                const float gsum = reduce_step<VB, G / 2>(gb, lane);
+                const int vb = val_of(G, VB, gl);
+                if (vb >= 0) put(vb, gsum);
+            } else {
+#pragma unroll
+                for (int i = 0; i < VB; ++i) {
+#pragma unroll
+                    for (int off = G / 2; off >= 1; off >>= 1) gb[i] += __shfl_xor_sync(kAll, gb[i], off);
+                    if (gl == i % G) put(i, gb[i]);
+                }
+            }
         }
     }
 }
 
-// Largest CTA of each variant: more points per thread need more registers.
-template <int R>
-constexpr int pts_max_threads() { return R <= 2 ? 384 : 256; }
+// Samples s0 .. s0 + count - 1 of one problem by the CTA's first `warps`
+// warps (all threads call it; the shared block is free again after the call).
+template <int G, int DIMS, int NF, bool WL, int TEAM>
+__device__ void pts_body(const ProjParams<float> &p, int s0, int count, int warps)
+{
+    float *sm = smem();
+    const PtsLayout L = pts_layout(G, DIMS, NF, p.nv, p.n_p, p.n_obs, p.n_static, warps, TEAM > 1 ? warps / TEAM : 0);
+    bool with_fix = false;
+    if constexpr (WL) {
+        unsigned dyn;
+        asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
+        with_fix = L.total_fix * sizeof(float) <= dyn;
+    }
+    if (threadIdx.x == 0) {
+        int *h = reinterpret_cast<int *>(sm);
+        h[kVrows] = int(L.vrows);
+        h[kNode] = int(L.node);
+        h[kTv] = int(L.tv);
+        h[kObs] = int(L.obs);
+        h[kObq] = int(L.obq);
+        h[kMov] = int(L.mov);
+        h[kGrid] = L.gsz && p.list_grid ? int(L.grid) : 0;
+        h[kFix] = with_fix ? int(L.fix) : 0;
+        h[kNp] = L.np;
+        h[kStamps] = p.n_p;
+        h[kStatic] = p.n_static;
+        h[kObstacles] = p.n_obs;
+        h[kNext] = (32 / G) * warps;
+        h[kXchAt] = int(L.xch);
+    }
+    if (threadIdx.x < 32) {
+        // node i of lane l: l mod G + i G
+        const float horizon = p.tab[p.lay.tval + p.n_p - 1];
+#pragma unroll
+        for (int i = 0; i < 32 / G; ++i) {
+            float2 r[NF + 1];
+            node_rows<NF>((threadIdx.x & (G - 1)) + i * G, horizon, r);
+#pragma unroll
+            for (int f = 0; f < (NF + 1) / 2; ++f)
+                reinterpret_cast<float4 *>(sm + L.node)[(i * ((NF + 1) / 2) + f) * 32 + threadIdx.x] =
+                    make_float4(r[2 * f].x, r[2 * f].y, r[2 * f + 1].x, r[2 * f + 1].y);
+        }
+    }
+    stage_tables<G, DIMS, NF, WL>(p, sm, L, with_fix);
+    const int warp = threadIdx.x >> 5, team = warp / TEAM, first = TEAM > 1 ? team : (32 / G) * warp;
+    const bool works = warp < warps && first < count;
+    Start<NF> start;
+    if (works) start = sample_start<G, DIMS, NF>(p, s0 + first, s0 + count);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (!works) return;
+    if constexpr (TEAM > 1) {
+        // (count is at most the number of teams)
+        project_samples<G, DIMS, NF, WL, TEAM>(p, int(L.warp0 + warp * L.wsz), s0 + team, s0 + count,
+                                               warp - TEAM * team, team, start);
+    } else {
+        // a warp's first samples by its number, then whichever are next
+        constexpr int NN = 32 / G;  // samples per warp
+        const int pw = int(L.warp0 + warp * L.wsz);
+        int i = first;
+        for (;;) {
+            project_samples<G, DIMS, NF, WL, 1>(p, pw, s0 + i, s0 + count, 0, 0, start);
+            if (NN * warps >= count) break;
+            if ((threadIdx.x & 31) == 0) i = atomicAdd(reinterpret_cast<int *>(sm) + kNext, NN);
+            i = __shfl_sync(kAll, i, 0);
+            if (i >= count) break;
+            start = sample_start<G, DIMS, NF>(p, s0 + i, s0 + count);
+        }
+    }
+}
 
-// The persistent form's CTA: the 2-D five-column variant with two points per
-// thread fits 128 registers, so two CTAs of 256 threads share an SM (16
-// warps; half the warps per barrier than one CTA of 512, and finer items);
-// the other variants keep one CTA of 384 per SM.  The single-problem launch
-// keeps the larger register budget, since its grid has one CTA per SM anyway.
-template <int DIMS, int R, int NF>
-constexpr int pts_batch_threads() { return (DIMS == 2 && R == 2 && NF == 5) ? 256 : pts_max_threads<R>(); }
-template <int DIMS, int R, int NF>
-constexpr int pts_batch_ctas_per_sm() { return (DIMS == 2 && R == 2 && NF == 5) ? 2 : 1; }
-
-template <int DIMS, int R, int NF, bool WL>
-__global__ void __launch_bounds__(pts_max_threads<R>(), 1) pts_kernel(const ProjParams<float> p)
+// One CTA per p.S samples; its first p.WS warps take them, all stage the tables.
+// (Teams of four leave an SM one CTA, so their warps may keep 255 registers.)
+template <int G, int DIMS, int NF, bool WL, int TEAM>
+__global__ void __launch_bounds__(32 * kMaxWarps, TEAM == 4 ? 1 : 2) pts_kernel(const ProjParams<float> p)
 {
     pdl_trigger();
     pdl_wait();
-    pts_body<DIMS, R, NF, WL>(p, blockIdx.x * p.S);
+    const int s0 = blockIdx.x * p.S;
+    pts_body<G, DIMS, NF, WL, TEAM>(p, s0, min(p.S, p.N - s0), p.WS);
 }
 
+// CTAs of the persistent form per SM that its registers allow.
+template <int DIMS, int NF>
+constexpr int pts_batch_ctas_per_sm() { return 2; }
+
 // Persistent form over many problems: CTAs take (problem, first sample)
-// items (each problem's p.S samples per item, p.S * TPS <= blockDim.x) through
-// an atomic counter until none is left; the item's parameters are staged in
-// shared memory (held in registers they would cost the CTA its size).  *next
-// must be zero at launch.
-template <int DIMS, int R, int NF, bool WL>
-__global__ void __launch_bounds__(pts_batch_threads<DIMS, R, NF>(), pts_batch_ctas_per_sm<DIMS, R, NF>())
+// items (p.S samples by p.WS warps) through an atomic counter until none is
+// left; the item's parameters are staged in shared memory.  *next must be zero
+// at launch.
+template <int G, int DIMS, int NF, bool WL>
+__global__ void __launch_bounds__(32 * kMaxWarps, pts_batch_ctas_per_sm<DIMS, NF>())
     pts_batch_kernel(const ProjParams<float> *params, const int2 *items, int n_items, int *next)
 {
     __shared__ int s_item;
@@ -1070,7 +1598,7 @@ __global__ void __launch_bounds__(pts_batch_threads<DIMS, R, NF>(), pts_batch_ct
         const int2 w = items[it];
         if (threadIdx.x == 0) s_p = params[w.x];
         __syncthreads();
-        pts_body<DIMS, R, NF, WL>(s_p, w.y);
+        pts_body<G, DIMS, NF, WL, 1>(s_p, w.y, min(s_p.S, s_p.N - w.y), s_p.WS);
         __syncthreads();
     }
 }

@@ -302,9 +302,18 @@ template <typename Real>
 cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vector<Slot *> &fresh, Stage &sg)
 {
     // ---- groups of the projection launch: same dims, free-coefficient count
-    //      and projection kernel
+    //      and projection kernel; the point-owner tilings of a group follow from
+    //      all its samples
     std::map<std::tuple<int, int, int>, std::vector<Slot *>> groups;
     for (Slot *s : active) groups[{s->h.sh.dims, s->h.sh.nf, s->t.kind}].push_back(s);
+    for (auto &g : groups) {
+        if (std::get<2>(g.first) != 1) continue;
+        std::vector<Shape> shapes;
+        for (Slot *s : g.second) shapes.push_back(s->h.sh);
+        std::vector<Tiling> tiles(shapes.size());
+        pts_batch_tiles(ctx, shapes, tiles);
+        for (size_t i = 0; i < tiles.size(); ++i) g.second[i]->t = tiles[i];
+    }
     // ---- layout of the staging block
     StepLayout lay;
     size_t o = 0;
