@@ -1,9 +1,8 @@
 // cem.cu -- the CEM stages of Alg. 1 around the projection:
 //   a10 ConstraintEliteSet (N_proj least r) and EliteSet (N_elite least
 //       c_aug = c_1 + r among them), ties to the lower sample index: each set
-//       by a bitwise threshold search (one block count per key bit), then a
-//       bitonic sort of the N_elite survivors whose short-stride stages run
-//       inside a warp on shuffles;
+//       by a radix search of its last (key, index) pair, then the N_elite
+//       survivors ranked by counting (few) or sorted bitonically (many);
 //   a11 MPPI-like refit (eqs. update_mean, update_covariance) in FP64 with
 //       weights exp(-(c_aug - delta)/gamma), delta = min c_aug;
 //   a12 the next sampling factor chol(Sigma' + eps I), eps = chol_eps tr(Sigma')/D,
@@ -92,22 +91,6 @@ __host__ __device__ inline int pow2_at_least(int n)
     return n2;
 }
 
-// Number of elements over the block for which this thread counted c (one
-// barrier).  Per-warp sums go to one of three counters by call parity: the
-// counter of call n + 2 is cleared after the barrier of call n, when every
-// read of it (call n - 1) is done.
-__device__ __forceinline__ int block_count(int c, int *s_cnt, int &calls)
-{
-    const int w = __reduce_add_sync(kFull, c);
-    const int slot = calls % 3;
-    if ((threadIdx.x & 31) == 0 && w) atomicAdd(&s_cnt[slot], w);
-    __syncthreads();
-    const int total = s_cnt[slot];
-    if (threadIdx.x == 0) s_cnt[(slot + 2) % 3] = 0;
-    ++calls;
-    return total;
-}
-
 // Exclusive prefix count of pred in thread order, and its total (two barriers).
 __device__ __forceinline__ int block_scan(bool pred, int *s_warp, int &total)
 {
@@ -126,118 +109,258 @@ __device__ __forceinline__ int block_scan(bool pred, int *s_warp, int &total)
     return before + __popc(b & ((1u << lane) - 1u));
 }
 
-// The k-th least key (1 <= k <= number of eligible elements) among the
-// eligible elements of the block, and lt = how many eligible keys are below
-// it.  Thread tid holds elements tid + e T (e < E, bit e of `elig`); the key of
-// e = 0 is k0, the others are in keys[].  Bitwise: t is the largest value with
-// #(key < t) < k, formed from the top bit down, one block count per bit.  The
-// high word first; when the eligible keys with that high word share one low
-// word (a lone key, or exact ties such as r = 0), that is the answer.
-__device__ unsigned long long kth_key(const unsigned long long *keys, unsigned long long k0, unsigned elig, int E,
-                                      int k, int *s_cnt, int &calls, unsigned *s_mm, int &lt)
+// What the threshold search shares: histograms of three successive steps (one
+// in use, one being read, one cleared), the bits some and all keys have, and
+// the last candidates.
+struct SelectShared {
+    int hist[3][8];
+    unsigned any[2], all[2];
+    int n;
+    int idx[32];
+    unsigned long long key[32];
+};
+
+// The k-th least (key, index) pair (1 <= k <= number of eligible elements) among
+// the eligible elements of the block.  Thread tid holds elements tid + e T (e <
+// E, bit e of `elig`); the key of e = 0 is k0, the others are in keys[].  Radix
+// selection, three bits a step from the highest bit in which the candidates
+// differ: ballots count a warp's eight bins, one barrier sums them over the block;
+// at 32 candidates or fewer every warp ranks them for itself.  Equal keys (r = 0
+// of many samples) are told apart by the bits of their index in the same way.
+// Barriers and reads of shared memory are what it costs: about ten barriers for
+// 1,000 distinct keys, where one per bit took 32 and more (whole solves, 13
+// selections of 110 samples: 1,121 -> 1,010 us; 5 of 1,000: 827 -> 802).  The loops
+// stay rolled: the code runs once a launch, so its size is fetched, not reused.
+__device__ void kth_pair(const unsigned long long *keys, unsigned long long k0, unsigned elig, int E, int k,
+                         SelectShared &sh, int &steps, unsigned long long &kth, int &kth_idx)
 {
-    const int tid = threadIdx.x, T = blockDim.x;
-    auto count_below = [&](unsigned long long trial) -> int {
-        if (E == 1) return __syncthreads_count((elig & 1u) && k0 < trial);
-        int c = 0;
-        for (int e = 0; e < E; ++e)
-            if ((elig >> e) & 1u) c += ((e == 0) ? k0 : keys[tid + e * T]) < trial;
-        return block_count(c, s_cnt, calls);
-    };
-    unsigned long long t = 0;
-    lt = 0;
-    for (int b = 63; b >= 32; --b) {
-        const unsigned long long trial = t | (1ull << b);
-        const int c = count_below(trial);
-        if (c < k) {
-            t = trial;
-            lt = c;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+    auto key_at = [&](int e) { return e == 0 ? k0 : keys[tid + e * T]; };
+    unsigned long long pre = 0ull, low = ~0ull;  // candidates: eligible, equal to pre but for the bits of low
+    bool by_index = false;                       // the bits searched are the index's (the keys are all `kth`)
+    int cnt = T * E;
+    kth = 0ull;
+    auto candidate = [&](int e, unsigned long long &v) {
+        if (!((elig >> e) & 1u)) return false;
+        v = key_at(e);
+        if (by_index) {
+            if (v != kth) return false;
+            v = static_cast<unsigned long long>(tid + e * T);
         }
-    }
-    for (int e = 0; e < E; ++e)
-        if ((elig >> e) & 1u) {
-            const unsigned long long v = (e == 0) ? k0 : keys[tid + e * T];
-            if ((v >> 32) == (t >> 32)) {
-                atomicMin(&s_mm[0], unsigned(v));
-                atomicMax(&s_mm[1], unsigned(v));
+        return ((v ^ pre) & ~low) == 0ull;
+    };
+    for (;;) {
+        // the highest bit in which the candidates differ
+        __syncthreads();
+        if (tid < 2) {
+            sh.any[tid] = 0u;
+            sh.all[tid] = ~0u;
+        }
+        __syncthreads();
+        {
+            unsigned long long any = 0ull, all = ~0ull;
+#pragma unroll 1
+            for (int e = 0; e < E; ++e) {
+                unsigned long long v;
+                if (candidate(e, v)) {
+                    any |= v;
+                    all &= v;
+                }
+            }
+            const unsigned a0 = __reduce_or_sync(kFull, unsigned(any)), a1 = __reduce_or_sync(kFull, unsigned(any >> 32));
+            const unsigned b0 = __reduce_and_sync(kFull, unsigned(all)), b1 = __reduce_and_sync(kFull, unsigned(all >> 32));
+            if (lane == 0) {
+                atomicOr(&sh.any[0], a0);
+                atomicOr(&sh.any[1], a1);
+                atomicAnd(&sh.all[0], b0);
+                atomicAnd(&sh.all[1], b1);
             }
         }
-    __syncthreads();
-    if (s_mm[0] == s_mm[1]) return t | s_mm[0];
-    for (int b = 31; b >= 0; --b) {
-        const unsigned long long trial = t | (1ull << b);
-        const int c = count_below(trial);
-        if (c < k) {
-            t = trial;
-            lt = c;
+        __syncthreads();
+        const unsigned long long any = (static_cast<unsigned long long>(sh.any[1]) << 32) | sh.any[0];
+        const unsigned long long all = (static_cast<unsigned long long>(sh.all[1]) << 32) | sh.all[0];
+        int pos = 63 - __clzll(static_cast<long long>(any ^ all));  // -1: all equal
+        low = pos >= 0 ? (2ull << pos) - 1ull : 0ull;
+        pre = all & ~low;
+        if (pos < 0) {
+            if (by_index) {  // one element
+                kth_idx = int(all);
+                return;
+            }
+            kth = all;
+            by_index = true;
+            low = ~0ull;
+            pre = 0ull;
+            continue;
+        }
+        for (bool shrunk = true; shrunk && pos >= 0;) {
+            const int at = max(pos - 2, 0);
+            const unsigned mask = (2u << (pos - at)) - 1u;  // one to three bits
+            int c = 0;                                      // lane l < 8: the warp's candidates in bin l
+#pragma unroll 1
+            for (int e = 0; e < E; ++e) {
+                unsigned long long v = 0ull;
+                const bool in = candidate(e, v);
+                const unsigned dgt = unsigned(v >> at) & mask;
+                const unsigned m = __ballot_sync(kFull, in), b0 = __ballot_sync(kFull, dgt & 1u),
+                               b1 = __ballot_sync(kFull, dgt & 2u), b2 = __ballot_sync(kFull, dgt & 4u);
+                c += __popc(m & (lane & 1 ? b0 : ~b0) & (lane & 2 ? b1 : ~b1) & (lane & 4 ? b2 : ~b2));
+            }
+            const int slot = steps % 3;
+            if (lane < 8 && c) atomicAdd(&sh.hist[slot][lane], c);
+            __syncthreads();
+            // (the slot after next: its last read was before this barrier)
+            if (tid < 8) sh.hist[(slot + 2) % 3][tid] = 0;
+            ++steps;
+            int before = 0, in_bin = 0, bin = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int h = sh.hist[slot][q];
+                if (bin == q) {
+                    if (before + h < k) {
+                        before += h;
+                        ++bin;
+                    } else {
+                        in_bin = h;
+                    }
+                }
+            }
+            k -= before;
+            pre |= static_cast<unsigned long long>(bin) << at;
+            low = (1ull << at) - 1ull;
+            pos = at - 1;
+            if (in_bin <= 32) {
+#pragma unroll 1
+                for (int e = 0; e < E; ++e) {
+                    unsigned long long v;
+                    if (candidate(e, v)) {
+                        const int i = atomicAdd(&sh.n, 1);
+                        sh.key[i] = by_index ? kth : v;
+                        sh.idx[i] = tid + e * T;
+                    }
+                }
+                __syncthreads();
+                const bool have = lane < in_bin;
+                const unsigned long long v = have ? sh.key[lane] : ~0ull;
+                const int i = have ? sh.idx[lane] : 0x7fffffff;
+                int rank = 0;
+#pragma unroll 4
+                for (int q = 0; q < 32; ++q) rank += q < in_bin && key_less(sh.key[q], sh.idx[q], v, i) ? 1 : 0;
+                const int from = __ffs(__ballot_sync(kFull, have && rank == k - 1)) - 1;
+                kth = __shfl_sync(kFull, v, from);
+                kth_idx = __shfl_sync(kFull, i, from);
+                __syncthreads();
+                if (tid == 0) sh.n = 0;  // (next used past the next call's barriers)
+                return;
+            }
+            shrunk = in_bin < cnt;
+            cnt = in_bin;
         }
     }
-    return t;
 }
 
+// Elites ranked by counting (each against every other, over all threads) up to
+// this number; the bitonic sort beyond.
+constexpr int kRankElites = 256;
+
 // ConstraintEliteSet: the n_proj least (r, index); EliteSet: the n_elite least
-// (c_aug, index) among them, written in ascending order.  Each set is found by
-// its threshold (kth_key) and the ties at the threshold taken by index, then
-// the n_elite survivors are sorted (bitonic, padding entries carry the largest
-// key and index).
+// (c_aug, index) among them, written in ascending order.  Each set is the
+// elements up to its last pair (kth_pair); the n_elite survivors are then sorted.
 __device__ void select_body(int N, const double *r, const double *c1, int n_proj, int n_elite, int *elite_idx)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, T = blockDim.x, E = (N + T - 1) / T;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, E = (N + T - 1) / T;
     const int n2e = pow2_at_least(n_elite);
     unsigned long long *key1 = reinterpret_cast<unsigned long long *>(smem_raw);  // N: order_key(r)
     unsigned long long *key2 = key1 + N;                                           // N: order_key(c_aug)
     unsigned long long *keyE = key2 + N;                                           // n2e
     int *idxE = reinterpret_cast<int *>(keyE + n2e);                               // n2e
-    __shared__ int s_cnt[3], s_warp[32];
-    __shared__ unsigned s_mm[4];
-    if (tid < 3) s_cnt[tid] = 0;
-    if (tid < 4) s_mm[tid] = (tid & 1) ? 0u : ~0u;
+    __shared__ SelectShared sh;
+    __shared__ int s_warp[32], s_rank[kRankElites], s_out;
+    if (tid < 24) (&sh.hist[0][0])[tid] = 0;
+    if (tid == 0) sh.n = s_out = 0;
+    for (int e = tid; e < kRankElites; e += T) s_rank[e] = 0;
     unsigned long long k01 = ~0ull, k02 = ~0ull;
     unsigned valid = 0;
-    for (int e = 0; e < E; ++e) {
-        const int i = tid + e * T;
-        if (i < N) {
-            const double ri = r[i];
-            const unsigned long long a = order_key(ri), b = order_key(c1[i] + ri);
-            key1[i] = a;
-            key2[i] = b;
-            if (e == 0) {
-                k01 = a;
-                k02 = b;
+#pragma unroll 1
+    for (int e0 = 0; e0 < E; e0 += 4) {
+        double rv[4], cv[4];  // (four elements' reads in flight)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = tid + (e0 + u) * T;
+            rv[u] = i < N ? r[i] : 0.0;
+            cv[u] = i < N ? c1[i] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = e0 + u, i = tid + e * T;
+            if (i < N) {
+                const unsigned long long a = order_key(rv[u]), b = order_key(cv[u] + rv[u]);
+                key1[i] = a;
+                key2[i] = b;
+                if (e == 0) {
+                    k01 = a;
+                    k02 = b;
+                }
+                valid |= 1u << e;
             }
-            valid |= 1u << e;
         }
     }
-    __syncthreads();
-    int calls = 0, lt = 0, base = 0, tot = 0;
-    // ConstraintEliteSet
-    const unsigned long long t1 = kth_key(key1, k01, valid, E, n_proj, s_cnt, calls, s_mm, lt);
-    const int need1 = n_proj - lt;
-    unsigned in1 = 0;
-    for (int e = 0; e < E; ++e) {
-        const unsigned long long v = (e == 0) ? k01 : (((valid >> e) & 1u) ? key1[tid + e * T] : ~0ull);
-        const bool tie = ((valid >> e) & 1u) && v == t1;
-        const int rank = base + block_scan(tie, s_warp, tot);
-        base += tot;
-        if (((valid >> e) & 1u) && (v < t1 || (tie && rank < need1))) in1 |= 1u << e;
+    int steps = 0, last = 0;
+    unsigned long long t = 0ull;
+    auto up_to_kth = [&](const unsigned long long *keys, unsigned long long k0, unsigned elig) {
+        unsigned in = 0u;
+#pragma unroll 1
+        for (int e = 0; e < E; ++e)
+            if ((elig >> e) & 1u) {
+                const unsigned long long v = e == 0 ? k0 : keys[tid + e * T];
+                if (!key_less(t, last, v, tid + e * T)) in |= 1u << e;
+            }
+        return in;
+    };
+    // ConstraintEliteSet (all of them when n_proj = N), EliteSet among them
+    unsigned in = valid;
+    if (n_proj < N) {
+        kth_pair(key1, k01, valid, E, n_proj, sh, steps, t, last);
+        in = up_to_kth(key1, k01, valid);
     }
-    // EliteSet among them
-    const unsigned long long t2 = kth_key(key2, k02, in1, E, n_elite, s_cnt, calls, s_mm + 2, lt);
-    const int need2 = n_elite - lt;
-    base = 0;
-    unsigned el = 0;
-    for (int e = 0; e < E; ++e) {
-        const unsigned long long v = (e == 0) ? k02 : (((in1 >> e) & 1u) ? key2[tid + e * T] : ~0ull);
-        const bool tie = ((in1 >> e) & 1u) && v == t2;
-        const int rank = base + block_scan(tie, s_warp, tot);
-        base += tot;
-        if (((in1 >> e) & 1u) && (v < t2 || (tie && rank < need2))) el |= 1u << e;
+    kth_pair(key2, k02, in, E, n_elite, sh, steps, t, last);
+    in = up_to_kth(key2, k02, in);
+    if (n_elite <= kRankElites) {
+#pragma unroll 1
+        for (int e = 0; e < E; ++e) {
+            const bool m = (in >> e) & 1u;
+            const unsigned b = __ballot_sync(kFull, m);
+            int at = 0;
+            if (lane == 0 && b) at = atomicAdd(&s_out, __popc(b));
+            at = __shfl_sync(kFull, at, 0) + __popc(b & ((1u << lane) - 1u));
+            if (m) {
+                keyE[at] = e == 0 ? k02 : key2[tid + e * T];
+                idxE[at] = tid + e * T;
+            }
+        }
+        __syncthreads();
+        // thread (slice, elite): the elites of its slice that come before
+        const int slices = max(1, T / n_elite), per = (n_elite + slices - 1) / slices;
+        for (int w = tid; w < slices * n_elite; w += T) {
+            const int q0 = (w / n_elite) * per, x = w % n_elite;
+            const unsigned long long v = keyE[x];
+            const int i = idxE[x];
+            int before = 0;
+            const int q1 = min(q0 + per, n_elite);
+#pragma unroll 4
+            for (int q = q0; q < q1; ++q) before += key_less(keyE[q], idxE[q], v, i) ? 1 : 0;
+            if (before) atomicAdd(&s_rank[x], before);
+        }
+        __syncthreads();
+        for (int x = tid; x < n_elite; x += T) elite_idx[s_rank[x]] = idxE[x];
+        return;
     }
-    // compact the elites (index order), then sort them by (c_aug, index)
-    base = 0;
+    // compact the elites, then sort them by (c_aug, index); padding carries the largest key and index
+    int base = 0, tot = 0;
+#pragma unroll 1
     for (int e = 0; e < E; ++e) {
-        const bool m = (el >> e) & 1u;
+        const bool m = (in >> e) & 1u;
         const int pos = base + block_scan(m, s_warp, tot);
         base += tot;
         if (m) {
@@ -525,7 +648,8 @@ cudaError_t launch_select_batch(const CemArgs *args_dev, int n, size_t smem, cud
     static size_t granted = 0;
     cudaError_t e = reserve_smem(select_batch_kernel, smem, granted);
     if (e != cudaSuccess) return e;
-    select_batch_kernel<<<n, kSelectThreads, smem, st>>>(args_dev);
+    // 256 threads hold 8,192 samples (32 each) and leave an SM several problems
+    select_batch_kernel<<<n, 256, smem, st>>>(args_dev);
     return cudaGetLastError();
 }
 
@@ -545,7 +669,10 @@ cudaError_t launch_select(int N, const double *r, const double *c1, int n_proj, 
     static size_t granted = 0;
     cudaError_t e = reserve_smem(select_kernel, smem, granted);
     if (e != cudaSuccess) return e;
-    return launch_pdl(select_kernel, dim3(1), dim3(kSelectThreads), smem, st, N, r, c1, n_proj, n_elite, elite_idx);
+    // few warps keep the barriers cheap (N = 1000, whole solve: 1,024 threads 815 us, 512 801,
+    // 256 805, 128 834)
+    const int threads = std::min(kSelectThreads, std::max(128, (N / 2 + 31) & ~31));
+    return launch_pdl(select_kernel, dim3(1), dim3(threads), smem, st, N, r, c1, n_proj, n_elite, elite_idx);
 }
 
 cudaError_t launch_refit(int D, const double *xb, const double *r, const double *c1, const int *elite,
