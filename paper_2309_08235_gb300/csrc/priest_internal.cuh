@@ -38,6 +38,8 @@ struct Shape {
     int cost_kind;                          // c_1: 0 = sum |a|^2; 1 = BARN-style
     double w_acc, w_curv, w_path, curv_eps;
     double list_delta;                      // neighbour-list margin (list_margin; 0 without obstacles)
+    double crowd;                           // share of the obstacles' bounding box that their discs fill
+    double grid_delta;                      // the largest margin the static-obstacle grid serves
 };
 
 // Neighbour-list margin of a problem (center: n_obs x dims, semi: n_obs x 2), 0
@@ -46,8 +48,13 @@ struct Shape {
 // shared inverse (W = (I + rho (n_obs P^T P + ...))^-1), so the denser the scene
 // the slower its trajectories move: the margin is such that the ball of radius
 // (mean largest semi-axis + margin) holds 0.25 obstacle centres on average at
-// the density of the centres' bounding box, kept between 1/4 and 5/2 of the
-// mean smallest semi-axis; 3/2 of it below 16 obstacles.
+// the density of the centres' bounding box, kept between 1/4 and 5/2 of the mean
+// smallest semi-axis; 3/2 of it below 16 obstacles.  The kernel doubles the margin
+// of lists that do not last; the static-obstacle grid serves (*grid_delta) at least
+// one mean semi-axis, so that it can (grids filled for the margin alone: 59 circles
+// in a small box, 81 samples, K = 52, 209 us a pass against 154; 41 circles, 2,026
+// samples 306 against 246; a least margin of 1 instead of 1/4 made 22 to 42 moving
+// circles on one corridor 1.4 to 1.8 times slower).
 // PRIEST_LIST_MARGIN=<multiple> sets the multiple instead (comparisons).
 inline double list_margin_scale()
 {
@@ -58,8 +65,10 @@ inline double list_margin_scale()
     return (end != v && x > 0.0 && x < 1e6) ? x : 0.0;
 }
 
-inline double list_margin(int dims, int n_obs, const double *center, const double *semi)
+inline double list_margin(int dims, int n_obs, const double *center, const double *semi, double *grid_delta,
+                          double *crowd)
 {
+    *grid_delta = *crowd = 0.0;
     if (n_obs <= 0) return 0.0;
     double s = 0.0, big = 0.0, lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
     for (int j = 0; j < n_obs; ++j) {
@@ -74,16 +83,21 @@ inline double list_margin(int dims, int n_obs, const double *center, const doubl
     }
     s /= n_obs;
     big /= n_obs;
-    const double scale = list_margin_scale();
-    if (scale > 0.0) return scale * s;
-    if (n_obs < 16) return 1.5 * s;
     double vol = 1.0;
     for (int ax = 0; ax < dims; ++ax) vol *= (hi[ax] - lo[ax]) + 2.0 * big;
     const double rho = n_obs / vol, pi = 3.141592653589793, held = 0.25;
+    *crowd = rho * (dims == 2 ? pi * big * big : 4.0 / 3.0 * pi * big * big * big);
+    const double scale = list_margin_scale();
+    *grid_delta = scale * s;
+    if (scale > 0.0) return scale * s;
+    *grid_delta = 1.5 * s;
+    if (n_obs < 16) return 1.5 * s;
     // radius of the ball that holds `held` centres on average
     const double r = dims == 2 ? __builtin_sqrt(held / (pi * rho)) : __builtin_cbrt(0.75 * held / (pi * rho));
-    const double delta = r - big;
-    return delta < 0.25 * s ? 0.25 * s : delta > 2.5 * s ? 2.5 * s : delta;
+    const double delta = r - big, least = 0.25 * s;
+    const double d = delta < least ? least : delta > 2.5 * s ? 2.5 * s : delta;
+    *grid_delta = d < s ? s : d;
+    return d;
 }
 
 // c_1 of the final pass (Alg. 1 cost): the point-to-point benchmark's
@@ -175,7 +189,7 @@ __host__ __device__ inline int fb_stride(int nf)
 // lists, in increasing order, the static obstacles whose screening disc (the
 // radius the inflated pre-filter can accept, plus slack) meets it; cells are
 // at least twice the largest such radius, so an obstacle meets at most 2 x 2
-// cells.  Region (4-byte units): header [x0, y0, 1/h, h, nx, ny, entries, 0]
+// cells.  Region (4-byte units): header [x0, y0, 1/h, h, nx, ny, entries, margin served]
 // (nx = 0: no grid), cell starts (uint16, nx * ny + 1), entries (uint16, at
 // most 4 per obstacle), then the set-up's per-obstacle cell ranges.
 constexpr int kGridMinStatic = 16;  // fewer static obstacles: screened directly

@@ -76,7 +76,12 @@ bool pts_allowed()
 template <typename Real>
 Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
 {
-    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed()) {
+    // Where many obstacles, almost all moving (no grid), fill half of their box with their discs,
+    // most pairs are active and the sums per time stamp of the chunked kernel are cheaper than
+    // the pairs' own (41 moving circles on a corridor, share 0.59, 755 samples: 123 against 216
+    // us; 22, share 0.35, the lists are faster; batched launches keep one kernel for all problems).
+    const bool crowded = sh.n_static < kGridMinStatic && sh.n_obs >= 32 && sh.crowd >= 0.5;
+    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed() && !crowded) {
         // an SM's share of the samples in as few CTAs of equal size as hold them
         const int m = std::max(1, (n_samples + n_sm - 1) / n_sm), G = pts_group(sh, m);
         // few samples per SM: a team of warps for each (pts_team_size)

@@ -74,6 +74,7 @@ constexpr int kMaxWarps = 8;    // warps of one CTA
 constexpr int kMaxStrides = 16; // strides of G time stamps
 constexpr int kPairs = 256;     // obstacle pairs a sample may list (a multiple of 32)
 constexpr int kShortLived = 6;  // iterations of a list that lasted too short
+constexpr int kRetry = 16;      // iterations without a list before the next try
 constexpr int kMaxTeam = 4;     // most warps of one sample's team
 // A team's exchange floats: two buffers of {sums of g [3][32], the test's answer}, {r^2, c_1}
 // [kMaxTeam][2] doubles, the fixed columns' sums [kMaxTeam][32]
@@ -432,10 +433,24 @@ struct Screen {
             unsigned m = __ballot_sync(kAll, may);
             if (G == 16) m = (m | (m >> 16)) & 0xffffu;  // either sample's
 #pragma unroll 1
-            for (; m; m &= m - 1) {
-                const int jm = j0 + __ffs(m) - 1;
-                const float4 o = pair_terms<DIMS>(jm, t, ns);
-                if (valid && near_pair<DIMS>(x, o, semi(jm), delta)) hit(jm, o);
+            while (m) {  // four at a time, their loads in flight together
+                int jm[4];
+                float4 o[4];
+                bool near[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    near[i] = valid && m != 0u;
+                    jm[i] = m ? j0 + __ffs(m) - 1 : j0;
+                    m &= m - 1u;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    o[i] = pair_terms<DIMS>(jm[i], t, ns);
+                    near[i] = near_pair<DIMS>(x, o[i], semi(jm[i]), delta) && near[i];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (near[i]) hit(jm[i], o[i]);
             }
         }
     }
@@ -1084,9 +1099,9 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     };
     // the warp's part of the rebuild, for every sample it holds.  Lists that lasted only a few
     // iterations are rebuilt with twice the margin, those of too many pairs with half of it
-    // (never beyond the margin that the grid's cells were filled for)
+    // (never beyond the margin that the grid's cells were filled for, in its header)
     float reach = delta;
-    const float widest = (hdr(kGrid) ? 1.f : 8.f) * delta;
+    const float widest = hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta;
     int built = -kShortLived;
     auto rebuild = [&](int need, int k, const float2 (&cc)[NF][DIMS]) {
         const bool need_p = need & 1, need_a = need & 2;
@@ -1099,13 +1114,16 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
                 for (;;) {
                     trips = build_list<TEAM>(gr, held, reach, role, team,
                                              reinterpret_cast<int *>(smem() + hdr(kXchAt) + team * kXch + kXchEnd));
-                    if (trips >= 0 || reach < 0.1f * delta) break;
+                    if (trips >= 0 || reach < 0.3f * delta) break;
                     reach *= 0.5f;
                 }
-                if (bounds && pos) mbx = wall_rows<G, DIMS, NF>(gr, p, reach);
+                if (trips < 0) reach = delta;
+                // (no list: nothing is tested, so every stride's workspace rows too)
+                if (bounds && pos) mbx = trips >= 0 ? wall_rows<G, DIMS, NF>(gr, p, reach) : (2u << ((n_p - 1) / G)) - 1u;
             }
-            // largest displacement between rebuilds: 7/8 of the margin (the rest covers rounding)
-            tauP2 = (0.875f / kNodeBoundPos) * reach * ((0.875f / kNodeBoundPos) * reach);
+            // largest displacement between rebuilds: 7/8 of the margin (the rest covers rounding);
+            // without a list every pair is screened, and a list tried again kRetry iterations on
+            tauP2 = trips >= 0 ? (0.875f / kNodeBoundPos) * reach * ((0.875f / kNodeBoundPos) * reach) : INFINITY;
         }
         if (need_a && (rate || tester)) {
             const RateRows rr = rate_rows<G, DIMS, NF>(gr, vmax, amax);
@@ -1134,6 +1152,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     }
     for (int k = 0, turn = 0;; ++k, ++turn) {
         load_coefs<DIMS, NF>(pc, c);
+        if (trips < 0 && lists && k - built >= kRetry) tauP2 = -1.f;
         // the pair that trip e of the list gives this lane: its residual and whether it is active
         auto trip = [&](int e, float (&r)[DIMS], int &t) {
             const float4 o = gr.list()[e * G + gl];
@@ -1253,7 +1272,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             for (int f = 0; f < (WL ? NB : 1); ++f)
 #pragma unroll
                 for (int ax = 0; ax < DIMS; ++ax) gf[f][ax] = gfix[f][ax];
-            dense_sums<G, DIMS, NF>(gr, delta, gg, WL ? gf : nullptr, p.tab + p.lay.basis, nv);
+            dense_sums<G, DIMS, NF>(gr, 0.f, gg, WL ? gf : nullptr, p.tab + p.lay.basis, nv);
             act = true;
 #pragma unroll
             for (int f = 0; f < NF; ++f)
@@ -1424,7 +1443,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             __syncwarp();
         }
     } else {
-        r2 += dense_squares<G, DIMS, NF>(gr, delta);
+        r2 += dense_squares<G, DIMS, NF>(gr, 0.f);
     }
     {
         // the lower half of the group ends with r2, the upper half with c_1

@@ -68,8 +68,8 @@ __device__ inline double screen_margin(double oo, double a, double kap, int dims
 
 // Step (9), FP32 tables: the uniform grid over the static obstacles (layout in
 // priest_internal.cuh) for the point-owner kernel's neighbour-list builds.
-// The pre-filter of the list build (thresholds inflated by the list margin
-// delta) accepts a point only within the x-y radius
+// The pre-filter of the list build (thresholds inflated by the largest list margin
+// that the grid serves, delta) accepts a point only within the x-y radius
 //   rho^2 = R^2 (1 + 1e-5) + 2 margin,  R = a + delta (2-D),
 //   R = a (1 + delta max(1/a, 1/b)) (3-D),
 // (the factor covers the FP32 evaluation of the expanded test and of the
@@ -99,7 +99,7 @@ __device__ void build_grid(const SetupParams &p, const double *org, float *reg, 
         }
         return;
     }
-    const float delta = float(sh.list_delta);
+    const float delta = float(sh.grid_delta);
     // centre (x, y) relative to the origin and screening radius of obstacle j
     auto geometry = [&](int j, float &cx, float &cy) {
         const float a = float(p.semi[2 * j]), b = dims == 3 ? float(p.semi[2 * j + 1]) : a;
@@ -258,7 +258,7 @@ __device__ void build_grid(const SetupParams &p, const double *org, float *reg, 
         reg[3] = s_geo[2];
         ireg[4] = nx;
         ireg[5] = ny;
-        ireg[7] = 0;
+        reg[7] = delta;
     }
 }
 

@@ -7,7 +7,7 @@ without any residual, and repeated samples, which only their index tells apart."
 import numpy as np
 import pytest
 
-from gpu_common import scene
+from gpu_common import TOL_FP64, rel_err, scale_of, scene
 from paper_2309_08235_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -44,3 +44,21 @@ def test_elites_are_the_sorted_prefix(P, N, n_proj, n_elite, ties):
     first = np.lexsort((i, r))[:n_proj]
     want = first[np.lexsort((first, (c1 + r)[first]))][:n_elite]
     np.testing.assert_array_equal(np.asarray(el), want)
+
+
+@pytest.mark.parametrize("N,n_elite", [(8192, 1024), (8161, 5), (300, 257)])
+def test_batched_selection_equals_the_single_one(P, N, n_elite):
+    """The batched launch's 256 threads hold up to 32 samples each; FP64 mode,
+    where both launches project to the same bits up to rounding."""
+    p = scene(n_obs=4, n_dyn=1, n_p=20)
+    cem = W.cem_settings(N, 2, 2, n_proj=max(n_elite, N // 2), n_elite=n_elite, dims=2)
+    z = W.normals(12, (2, N, 22))
+    with P.Context(p, cem, precision=P.PRIEST_FP64_CHECK, autotune=0) as ctx:
+        one = ctx.plan(p, z=z)
+        struct, keep = P.make_problem(p, cem, per_problem_shape=True)
+        res = (P.priest_result * 1)()
+        P.priest_plan_batch_host(ctx.h, [struct], [z], res)
+        both = P.result_dict(res[0])
+    assert both["best_index"] == one["best_index"]
+    assert rel_err(both["best"], one["best"], scale_of(p)) < TOL_FP64
+    assert rel_err(both["mu"], one["mu"], scale_of(p)) < TOL_FP64
