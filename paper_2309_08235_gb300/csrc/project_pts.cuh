@@ -981,8 +981,10 @@ __device__ __forceinline__ Start<NF> sample_start(const ProjParams<float> &p, in
 // and role 3 makes the node test beside them; of two, role 1 does both.  The
 // partial sums of g and the test's answer meet in shared memory (one barrier an
 // iteration); when the lists no longer hold, the sums are dropped, the lists
-// rebuilt (a stride of time stamps to a warp) and the iteration done again.  Every
-// warp repeats the multiplier and shared-inverse steps.
+// rebuilt (a stride of time stamps to a warp) and the iteration done again, once:
+// lists just built hold, and are not tested, so an iteration takes at most two
+// passes whatever the test's arithmetic makes of its inputs.  Every warp repeats the
+// multiplier and shared-inverse steps.
 template <int G, int DIMS, int NF, bool WL, int TEAM>
 __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int pw, int s_first, int s_end, int role,
                                                 int team, const Start<NF> &start)
@@ -1145,10 +1147,12 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
                 }
             }
     };
+    bool fresh = false;  // the lists were built for this iteration's coefficients (the same in all of a team)
     if (TEAM > 1 && lists) {
         float2 cc[NF][DIMS];
         load_coefs<DIMS, NF>(pc, cc);
         rebuild(3, 0, cc);
+        fresh = true;
     }
     for (int k = 0, turn = 0;; ++k, ++turn) {
         load_coefs<DIMS, NF>(pc, c);
@@ -1173,7 +1177,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             if (pos) {
                 in0 = trip(0, r0, t0);
             }
-            if (tester) {
+            if (tester && !fresh) {
                 float2 cc[NF][DIMS];
                 load_coefs<DIMS, NF>(pc, cc);
                 need = outdated(cc);
@@ -1361,7 +1365,8 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
                         for (int ax = 0; ax < DIMS; ++ax) gfix[f][ax] = gfix0[f][ax];
             }
             if (last) break;
-            if (need != 0) {
+            fresh = need != 0;
+            if (fresh) {
                 --k;
                 continue;
             }
