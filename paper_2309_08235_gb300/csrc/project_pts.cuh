@@ -17,10 +17,14 @@
 // Position and acceleration are polynomials of degree 10 and 8 in time, and a
 // polynomial of degree n is bounded on its interval by 1 / cos(n pi / 2m) times
 // its maximum over m Chebyshev nodes (Ehlich and Zeller 1964).  The lanes
-// evaluate the displacement of 32 nodes since the last rebuild; while the bound
-// stays below the margins, every pair and row left out is inactive.  (The start's
-// velocity is fixed, so the change of velocity is bounded by that of the
-// acceleration times the time.)  Nothing is approximated: the sums are bitwise
+// evaluate the displacement of 32 nodes since the last rebuild, from the
+// coefficients' differences (which keep their digits wherever the frame's origin
+// lies); while the bound stays below the margins, every pair and row left out is
+// inactive.  (The start's velocity is fixed, so the change of velocity is bounded by
+// that of the acceleration times the time.)  The margins also pay for the rounding of
+// the rows, which grows with the coefficients (row_rounding): far from the origin the
+// lists shrink what may move before a rebuild, and where rounding alone eats the
+// margin every pair is screened.  So nothing is approximated: the sums are bitwise
 // those of evaluating every pair.  The m-th active pair in (t, j) order is added
 // by lane m mod G, whatever was listed beside it, and velocity, acceleration and
 // workspace rows by the owner of t, in a fixed order.
@@ -84,7 +88,7 @@ constexpr int kXchFlag = 3 * 32, kXchBuf = kXchFlag + 8, kXchEnd = 2 * kXchBuf, 
 // Shared-memory layout (float units, every block 32-byte aligned); np is n_p
 // rounded up to 2 G and the row blocks are arrays of 16 bytes over the stamps, so
 // the lanes of a group read neighbouring banks.
-//   header [16]               ints: the offsets and sizes below (Hdr)
+//   header [24]               ints: the offsets and sizes below (Hdr); floats: the origin, the extent, 1 / T
 //   rows  [chunks][np][4]     per time stamp, positions: nf free columns of P, then the
 //                             fixed-coefficient part of each axis
 //   vrows [2][pchunks][np / 2][4]  the same of Pd and Pdd, stamps 2 u and 2 u + 1
@@ -100,13 +104,19 @@ constexpr int kXchFlag = 3 * 32, kXchBuf = kXchFlag + 8, kXchEnd = 2 * kXchBuf, 
 //     stage [4 G][4]          active pairs on their way to a lane: {r (dims), t}
 //     list [kPairs][4]        2-D {1/a, -o_x(t)/a, -o_y(t)/a, a}, 3-D {1/a, -o_x(t)/a, -o_y(t)/a, -o_z(t)/b}
 //     tj [kPairs]             (ints) time stamp | obstacle << 16
+//     moved [nf][dims][2]     coefficients since the rebuild of the {pair, rate} lists
 //   xch   [teams][kXch]       what a team's warps tell one another
 //   fix   [3][fchunks][np][4] fixed columns (multipliers on request, when it fits)
-constexpr int kRows = 16;  // offset of the rows
+constexpr int kRows = 24;  // offset of the rows
+constexpr int kOrigin = 16, kExtent = 19, kRate = 20;  // of the header's floats (kRate: 1 / horizon)
 __host__ __device__ constexpr int coef_floats(int dims, int nf) { return nf * (dims == 2 ? 4 : 8); }
-__host__ __device__ constexpr int sample_floats(int G, int dims, int nf)
+__host__ __device__ constexpr int moved_at(int G, int dims, int nf)
 {
     return coef_floats(dims, nf) + 16 * G + 5 * kPairs + (nf & 1) * 4;
+}
+__host__ __device__ constexpr int sample_floats(int G, int dims, int nf)
+{
+    return (moved_at(G, dims, nf) + 2 * nf * dims + 7) & ~7;
 }
 struct PtsLayout {
     int np, nch, pch, nfch;
@@ -604,6 +614,7 @@ struct Group {
     }
     __device__ __forceinline__ float4 *list() const { return stage() + 4 * G; }
     __device__ __forceinline__ int *tj() const { return reinterpret_cast<int *>(list() + kPairs); }
+    __device__ __forceinline__ int moved() const { return pc + moved_at(G, DIMS, NF); }
 };
 
 // The sample's coefficients, each in both halves of a register pair.
@@ -628,6 +639,42 @@ __device__ __forceinline__ void load_coefs(int pc, float (&c)[NF][DIMS])
     for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int ax = 0; ax < DIMS; ++ax) c[f][ax] = d[f][ax].x;
+}
+
+// What rounding can make of the difference between two evaluations of a sample's
+// rows (positions, velocities, accelerations; the larger of a warp's two samples).
+// A row is a chain of NF FMAs that starts at its fixed part, and each rounds by at
+// most u = 2^-24 of its partial sum: the result less the terms to come, so at most
+// |result| + (sum of their |columns|) max |c|.  The columns' part, summed over the
+// chain and the largest over the horizon, is kappa: 2.13, 9.54 / T, 81.4 / T^2 with
+// five free columns, 4.25, 60 / T, 1530 / T^2 with seven.  A position is a mean of the
+// coefficients (Bernstein), so at most the largest one's distance from the origin.
+struct Rounding {
+    float pos, vel, acc;
+};
+template <int G, int DIMS, int NF>
+__device__ __forceinline__ Rounding row_rounding(const float2 (&c)[NF][DIMS], float vmax, float amax)
+{
+    static_assert(NF == 5 || NF == 7, "kappa");
+    float most = 0.f, extent = smem()[kExtent];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int ax = 0; ax < DIMS; ++ax) {
+            most = fmaxf(most, fabsf(c[f][ax].x));
+            extent = fmaxf(extent, fabsf(c[f][ax].x - smem()[kOrigin + ax]));
+        }
+    if (G == 16) {
+        most = fmaxf(most, __shfl_xor_sync(kAll, most, 16));
+        extent = fmaxf(extent, __shfl_xor_sync(kAll, extent, 16));
+    }
+    const float w = most * smem()[kRate], w2 = w * smem()[kRate];
+    constexpr float two = 2.f * (DIMS == 2 ? 1.4143f : 1.7321f) * 5.9605e-8f;  // evaluations, axes
+    Rounding r;
+    r.pos = two * fmaf(NF == 5 ? 2.2f : 4.3f, most, (NF + 1) * extent);
+    r.vel = two * fmaf(NF == 5 ? 9.6f : 60.f, w, (NF + 1) * vmax);
+    r.acc = two * fmaf(NF == 5 ? 82.f : 1530.f, w2, (NF + 1) * amax);
+    return r;
 }
 
 // The scaled offset of the pair with the terms o (3-D: obstacle j), its square
@@ -870,7 +917,8 @@ __device__ __forceinline__ RateRows rate_rows(Group<G, DIMS, NF> gr, float vmax,
     // the velocity changes by at most `reach` times what the acceleration does (NF = 5: it is
     // fixed at both ends)
     const float reach = (NF == 5 ? 0.5f : 1.f) * smem()[hdr(kTv) + hdr(kStamps) - 1];
-    const float slv = 0.95f * (vmax - sqrtf(v2)), sla = 0.95f * (amax - sqrtf(a2));
+    const Rounding rd = row_rounding<G, DIMS, NF>(c, vmax, amax);
+    const float slv = 0.95f * (vmax - sqrtf(v2)) - rd.vel, sla = 0.95f * (amax - sqrtf(a2)) - rd.acc;
     const unsigned all = (1u << (np / (2 * G))) - 1u;
     float da = fminf(sla, slv / reach);
     unsigned vel = 0u, acc = 0u;
@@ -880,7 +928,7 @@ __device__ __forceinline__ RateRows rate_rows(Group<G, DIMS, NF> gr, float vmax,
     }
     if (!(sla >= da)) {
         // blocks with an acceleration within the margin (a NaN counts as within)
-        const float la = fmaxf(0.f, amax - 1.05f * da), la2 = la * la;
+        const float la = fmaxf(0.f, amax - 1.05f * da - rd.acc), la2 = la * la;
 #pragma unroll 1
         for (int u = gr.gl, i = 0; u < np / 2; u += G, ++i) {
             float2 row[NF], a[DIMS];
@@ -1017,8 +1065,11 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
 #pragma unroll
     for (int f = 0; f < NF; ++f) wrow[f] = start.wrow[f];
     float2 *stp = reinterpret_cast<float2 *>(smem() + pc + sf * CS + 2 * sax);  // this lane's coefficient
+    float2 *stm = reinterpret_cast<float2 *>(smem() + gr.moved()) + sf * DIMS + sax;
+    float refP = stC, refA = stC;  // the coefficient at the last rebuild of the pair and rate lists
     __syncwarp();
     if (stv) *stp = make_float2(stC, stC);
+    if (stv) *stm = make_float2(0.f, 0.f);
     gr.list()[gl] = make_float4(0.f, 4.f, 0.f, 0.f);  // (evaluated once before the first rebuild)
     gr.tj()[gl] = 0;
     __syncwarp();
@@ -1037,11 +1088,6 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             if (2 * f + 1 <= NF) node[2 * f + 1] = make_float2(v.z, v.w);
         }
     };
-    float2 ref[NN][DIMS];  // node displacement {position, acceleration} = ref + node . c
-#pragma unroll
-    for (int i = 0; i < NN; ++i)
-#pragma unroll
-        for (int ax = 0; ax < DIMS; ++ax) ref[i][ax] = make_float2(0.f, 0.f);
     // a negative threshold makes the first iteration build
     float tauP2 = lists ? -1.f : INFINITY, tauA2 = tauP2;
     int trips = lists ? 1 : -1;  // of the pair list (the longest of the warp); -1: screen every time stamp
@@ -1080,18 +1126,30 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     float c[NF][DIMS];
     // which lists the nodes' displacement since the last rebuild no longer proves: bit 0 the
     // positions', bit 1 the rates'
-    auto outdated = [&](const float2 (&cc)[NF][DIMS]) {
+    auto outdated = [&]() {
         float e_p = 0.f, e_a = 0.f;  // its square
+        float2 m[NF][DIMS];
+#pragma unroll
+        for (int f = 0; f < NF * DIMS; f += 2) {
+            const int at = gr.moved() + 2 * f;
+            if (f + 1 < NF * DIMS) {
+                const float4 v = ld4s(at);
+                m[f / DIMS][f % DIMS] = make_float2(v.x, v.y);
+                m[(f + 1) / DIMS][(f + 1) % DIMS] = make_float2(v.z, v.w);
+            } else {
+                m[f / DIMS][f % DIMS] = *reinterpret_cast<const float2 *>(smem() + at);
+            }
+        }
 #pragma unroll
         for (int i = 0; i < NN; ++i) {
             float2 e[DIMS], node[NF + 1];
             load_node(i, node);
 #pragma unroll
-            for (int ax = 0; ax < DIMS; ++ax) e[ax] = ref[i][ax];
+            for (int ax = 0; ax < DIMS; ++ax) e[ax] = fmul2(node[0], m[0][ax]);
 #pragma unroll
-            for (int f = 0; f < NF; ++f)
+            for (int f = 1; f < NF; ++f)
 #pragma unroll
-                for (int ax = 0; ax < DIMS; ++ax) e[ax] = ffma2(node[f], cc[f][ax], e[ax]);
+                for (int ax = 0; ax < DIMS; ++ax) e[ax] = ffma2(node[f], m[f][ax], e[ax]);
             const float2 n = norm2<DIMS>(e);
             e_p = fmaxf(e_p, n.x);
             e_a = fmaxf(e_a, n.y);
@@ -1101,19 +1159,29 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     };
     // the warp's part of the rebuild, for every sample it holds.  Lists that lasted only a few
     // iterations are rebuilt with twice the margin, those of too many pairs with half of it
-    // (never beyond the margin that the grid's cells were filled for, in its header)
+    // (never beyond the margin that the grid's cells were filled for, in its header); rounding
+    // may take two fifths of a margin
     float reach = delta;
     const float widest = hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta;
     int built = -kShortLived;
-    auto rebuild = [&](int need, int k, const float2 (&cc)[NF][DIMS]) {
+    auto rebuild = [&](int need, int k) {
         const bool need_p = need & 1, need_a = need & 2;
         if (need_p) {
+            float rounding;
+            {
+                float2 cc[NF][DIMS];
+                load_coefs<DIMS, NF>(pc, cc);
+                rounding = row_rounding<G, DIMS, NF>(cc, vmax, amax).pos;
+            }
             if (k - built < kShortLived) reach = fminf(2.f * reach, widest);
+            reach = fmaxf(reach, fminf(4.f * rounding, widest));
             built = k;
+            refP = stC;
             if (pos || TEAM > 1) {
                 Group<G, DIMS, NF> held = gr;  // role 0's block holds the list
                 held.pc -= role * sample_floats(G, DIMS, NF);
-                for (;;) {
+                trips = -1;
+                while (rounding <= 0.4f * reach) {
                     trips = build_list<TEAM>(gr, held, reach, role, team,
                                              reinterpret_cast<int *>(smem() + hdr(kXchAt) + team * kXch + kXchEnd));
                     if (trips >= 0 || reach < 0.3f * delta) break;
@@ -1123,35 +1191,22 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
                 // (no list: nothing is tested, so every stride's workspace rows too)
                 if (bounds && pos) mbx = trips >= 0 ? wall_rows<G, DIMS, NF>(gr, p, reach) : (2u << ((n_p - 1) / G)) - 1u;
             }
-            // largest displacement between rebuilds: 7/8 of the margin (the rest covers rounding);
-            // without a list every pair is screened, and a list tried again kRetry iterations on
-            tauP2 = trips >= 0 ? (0.875f / kNodeBoundPos) * reach * ((0.875f / kNodeBoundPos) * reach) : INFINITY;
+            // largest displacement between rebuilds: 7/8 of the margin (the rest covers the rounding
+            // of the tests) less that of the rows; without a list every pair is screened, and a list
+            // tried again kRetry iterations on
+            const float far = fmaf(0.875f / kNodeBoundPos, reach, -rounding);
+            tauP2 = trips >= 0 ? far * far : INFINITY;
         }
+        if (need_a) refA = stC;
         if (need_a && (rate || tester)) {
             const RateRows rr = rate_rows<G, DIMS, NF>(gr, vmax, amax);
             rates = rr.bits & rate_mask;
             tauA2 = rr.tau2;
         }
-        if (TEAM == 1 || tester)
-#pragma unroll
-            for (int i = 0; i < NN; ++i) {
-                float2 node[NF + 1];
-                load_node(i, node);
-#pragma unroll
-                for (int ax = 0; ax < DIMS; ++ax) {
-                    float2 e = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int f = 0; f < NF; ++f) e = ffma2(make_float2(-node[f].x, -node[f].y), cc[f][ax], e);
-                    if (need_p) ref[i][ax].x = e.x;
-                    if (need_a) ref[i][ax].y = e.y;
-                }
-            }
     };
     bool fresh = false;  // the lists were built for this iteration's coefficients (the same in all of a team)
     if (TEAM > 1 && lists) {
-        float2 cc[NF][DIMS];
-        load_coefs<DIMS, NF>(pc, cc);
-        rebuild(3, 0, cc);
+        rebuild(3, 0);
         fresh = true;
     }
     for (int k = 0, turn = 0;; ++k, ++turn) {
@@ -1177,11 +1232,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             if (pos) {
                 in0 = trip(0, r0, t0);
             }
-            if (tester && !fresh) {
-                float2 cc[NF][DIMS];
-                load_coefs<DIMS, NF>(pc, cc);
-                need = outdated(cc);
-            }
+            if (tester && !fresh) need = outdated();
             if constexpr (WL)
 #pragma unroll
                 for (int f = 0; f < NB; ++f)
@@ -1192,11 +1243,9 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             for (bool tested = false;; tested = true) {
                 in0 = trip(0, r0, t0);
                 if (tested) break;
-                float2 cc[NF][DIMS];
-                load_coefs<DIMS, NF>(pc, cc);
-                need = outdated(cc);
+                need = outdated();
                 if (need == 0) break;
-                rebuild(need, k, cc);
+                rebuild(need, k);
             }
             if (k == K) break;
         }
@@ -1355,9 +1404,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
             team_sync<TEAM>(team);
             need = __float_as_int(x[kXchFlag]);
             if (need != 0) {
-                float2 cc[NF][DIMS];
-                load_coefs<DIMS, NF>(pc, cc);
-                rebuild(need, k, cc);
+                rebuild(need, k);
                 if constexpr (WL)
 #pragma unroll
                     for (int f = 0; f < NB; ++f)
@@ -1380,7 +1427,10 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
         float du = 0.f;
         gather_u<G, DIMS, NF, 0>(u, src0, wrow, du);
         stC += du;
-        if (stv) *stp = make_float2(stC, stC);
+        if (stv) {
+            *stp = make_float2(stC, stC);
+            *stm = make_float2(stC - refP, stC - refA);
+        }
         __syncwarp();
     }
 
@@ -1562,6 +1612,21 @@ __device__ void pts_body(const ProjParams<float> &p, int s0, int count, int warp
         }
     }
     stage_tables<G, DIMS, NF, WL>(p, sm, L, with_fix);
+    if (threadIdx.x >= 32 * (kMaxWarps - 1)) {
+        // the origin, the fixed coefficients' largest distance from it, 1 / T (the last warp: the
+        // first ones have samples to start; read beside the staging)
+        const int lane = threadIdx.x & 31;
+        float e = 0.f;
+        for (int d = lane; d < DIMS * p.nv; d += 32) {
+            const int ax = d / p.nv, col = d - ax * p.nv;
+            if (col < kFree0 || col >= kFree0 + NF)
+                e = fmaxf(e, float(fabs(p.cB[ax * kMaxNv + col] - double(p.tab[p.lay.origin + ax]))));
+        }
+        e = __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(e)));
+        if (lane == 0) sm[kExtent] = e;
+        if (lane == 0) sm[kRate] = 1.f / p.tab[p.lay.tval + p.n_p - 1];
+        if (lane < DIMS) sm[kOrigin + lane] = p.tab[p.lay.origin + lane];
+    }
     const int warp = threadIdx.x >> 5, team = warp / TEAM, first = TEAM > 1 ? team : (32 / G) * warp;
     const bool works = warp < warps && first < count;
     Start<NF> start;

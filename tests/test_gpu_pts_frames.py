@@ -1,8 +1,9 @@
 """The FP32 point-owner projection far from the frame's origin, with outlying
 coefficients and with a margin below FP32's resolution: where coefficients round
 coarsely the node test's own rounding can exceed its threshold, and an iteration
-must still be done at most twice.  Teams of four and of two warps per sample, one
-warp, and two samples per warp."""
+must still be done at most twice, with bitwise the results of screening every pair
+in every iteration.  Teams of four and of two warps per sample, one warp, and two
+samples per warp."""
 import os
 
 import numpy as np
@@ -26,6 +27,12 @@ def shifted(p, off):
     return q
 
 
+def same(a, b):
+    for x, y in zip(a, b):
+        if x is not None:
+            np.testing.assert_array_equal(x, y)
+
+
 @pytest.mark.parametrize("dims,mask", [(2, 7), (3, 7), (2, 1)])
 @pytest.mark.parametrize("form", list(PER_SM))
 @pytest.mark.parametrize("off,horizon", [(1e4, 6.0), (1e5, 1.0), (1e5, 6.0), (5e5, 2.0), (4.6e6, 5.0)])
@@ -38,7 +45,9 @@ def test_far_frames(P, oracle, off, horizon, form, dims, mask):  # noqa: F811
     p = shifted(scene(dims=dims, n_obs=24, n_dyn=3, n_p=60, horizon=horizon, mask=mask, amax=1.5), off)
     n = PER_SM[form] * sm_count() - 3
     xi = samples(oracle, p, n, seed=3)
-    xb, _, r, _ = project(P, p, xi, K, None, "1")
+    got = project(P, p, xi, K, None, "1")
+    same(got, project(P, p, xi, K, None, "0"))
+    xb, _, r, _ = got
     assert np.isfinite(xb).all() and np.isfinite(r).all()
     if off * (6.0 / horizon) ** 2 <= 1e5:
         idx = np.r_[0:n:max(1, n // 9), n - 1]
@@ -57,6 +66,7 @@ def test_outlying_coefficients(P, oracle, value, form, dims, mask):  # noqa: F81
     odd = xi.copy()
     odd[::5, 5] = value
     a = project(P, p, odd, K, None, "1")
+    same(a, project(P, p, odd, K, None, "0"))
     b = project(P, p, xi, K, None, "1")
     rest = np.arange(n) % 5 != 0
     for x, y in zip(a, b):
@@ -75,7 +85,4 @@ def test_margin_below_resolution(P, oracle, form, dims, mask):  # noqa: F811
         a = project(P, p, xi, K, None, "1")
     finally:
         os.environ.pop("PRIEST_LIST_MARGIN")
-    b = project(P, p, xi, K, None, "0")
-    for x, y in zip(a, b):
-        if x is not None:
-            np.testing.assert_array_equal(x, y)
+    same(a, project(P, p, xi, K, None, "0"))
