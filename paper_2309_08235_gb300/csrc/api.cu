@@ -1716,7 +1716,7 @@ priest_status project_batch(priest_ctx *ctx, int n, priest_loaded *const *probs,
     int kind = 0, R = 4;
     s = batch_tiles<Real>(ctx, shapes, tiles, kind, R);
     if (s != PRIEST_OK) return s;
-    size_t smem = 0;
+    size_t smem = 0, smem_fix = 0;
     std::vector<std::pair<double, int2>> items;
     ProjParams<Real> *hp = reinterpret_cast<ProjParams<Real> *>(hb + o_par);
     for (int i = 0; i < n; ++i) {
@@ -1726,10 +1726,12 @@ priest_status project_batch(priest_ctx *ctx, int n, priest_loaded *const *probs,
         p.WS = tiles[i].ws;
         hp[i] = p;
         smem = std::max(smem, tiles[i].smem);
+        smem_fix = std::max(smem_fix, tiles[i].smem_fix);
         const double cost = double(shapes[i].n_p) * (double(shapes[i].n_obs) + 12.0);
         for (int s0 = 0; s0 < rows[i]; s0 += tiles[i].S)
             items.push_back({cost * std::min(tiles[i].S, rows[i] - s0), make_int2(i, s0)});
     }
+    if (kind == 1 && want_lambda) smem = pts_batch_smem(smem, smem_fix, int(items.size()));
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, int2> &x, const std::pair<double, int2> &y) { return x.first > y.first; });
     int2 *hi = reinterpret_cast<int2 *>(hb + o_it);

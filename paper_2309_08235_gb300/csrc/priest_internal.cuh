@@ -325,6 +325,7 @@ struct Tiling {
     int ws;       // warps per sample (chunked) / warps of the CTA that take samples (point-owner)
     size_t smem;  // dynamic shared memory bytes
     int kind = 0; // 0: chunked kernel (project_kernel.cuh); 1: point-owner FP32 kernel (project_pts.cuh)
+    size_t smem_fix = 0;  // point-owner: smem with the fixed columns' rows of a launch that returns multipliers
 };
 
 // FP32 point-owner kernel (project_pts.cu): degree 10 with 5 free coefficients
@@ -336,6 +337,8 @@ Tiling pts_tiling(const Shape &sh, int G, int warps);  // 32 / G samples per war
 int pts_team_size(const Shape &sh, int samples_per_sm);  // warps per sample of a team, 0: no team
 Tiling pts_team_tiling(const Shape &sh, int teams, int C);  // teams of C warps, a sample each
 Tiling pts_batch_tiling(const Shape &sh, int G, int samples_per_sm);  // item of the persistent launch
+// Shared memory of a persistent launch that returns multipliers (smem, smem_fix: the largest of its problems)
+size_t pts_batch_smem(size_t smem, size_t smem_fix, int n_items);
 
 // Raises a kernel's dynamic shared-memory limit to `bytes` (the default limit
 // counts static shared memory too, so it is raised whenever more is asked

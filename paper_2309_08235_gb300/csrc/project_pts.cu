@@ -9,20 +9,26 @@ namespace priest {
 
 namespace {
 
-constexpr size_t kSmemCap = 227 * 1024;
-// Shared memory of one CTA when two share an SM (228 KB less 1 KB and the
-// static part of each).
-constexpr size_t kSmemHalf = 112 * 1024;
+using pts::kSmemCap;
+using pts::kSmemHalf;
 // Samples one warp takes per item of the persistent launch: enough to bury
 // the staging of the item's tables, few enough for an even end.
 constexpr int kSamplesPerWarp = 4;
 
 }  // namespace
 
+namespace {
+
+pts::PtsLayout layout_of(const Shape &sh, int G, int warps, int C)
+{
+    return pts::pts_layout(G, sh.dims, sh.nf, sh.nv, sh.n_p, sh.n_obs, sh.n_static, warps, C > 1 ? warps / C : 0);
+}
+
+}  // namespace
+
 size_t pts_smem_bytes(const Shape &sh, int G, int warps, int C)
 {
-    return pts::pts_layout(G, sh.dims, sh.nf, sh.nv, sh.n_p, sh.n_obs, sh.n_static, warps, C > 1 ? warps / C : 0).total *
-           sizeof(float);
+    return layout_of(sh, G, warps, C).total * sizeof(float);
 }
 
 // Degree 10 with the "at rest" end (5 free coefficients per axis), 2-D or
@@ -48,6 +54,7 @@ Tiling pts_tiling(const Shape &sh, int G, int warps)
     t.S = w * (32 / G);
     t.threads = 32 * pts::kMaxWarps;
     t.smem = pts_smem_bytes(sh, G, w, 1);
+    t.smem_fix = layout_of(sh, G, w, 1).total_fix * sizeof(float);
     if (!pts_supported(sh) || t.smem > kSmemCap) t.smem = 0;
     return t;
 }
@@ -78,6 +85,7 @@ Tiling pts_team_tiling(const Shape &sh, int teams, int C)
     t.S = teams;
     t.threads = 32 * pts::kMaxWarps;
     t.smem = pts_smem_bytes(sh, 32, t.ws, t.C);
+    t.smem_fix = layout_of(sh, 32, t.ws, t.C).total_fix * sizeof(float);
     if (!pts_supported(sh) || t.ws > pts::kMaxWarps || t.smem > kSmemCap) t.smem = 0;
     return t;
 }
@@ -110,19 +118,23 @@ Tiling pts_batch_tiling(const Shape &sh, int G, int samples_per_sm)
 
 namespace {
 
-// Bytes of the fixed columns' rows, added to launches that return
-// multipliers when they fit (they are read from global memory otherwise).
-size_t fix_bytes(int n_p, int nf) { return size_t(3) * ((11 - nf + 3) / 4) * ((n_p + 31) & ~31) * 16; }
+int sm_count()
+{
+    int dev = 0, n_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    return n_sm;
+}
 
 template <int G, int DIMS, int NF, bool WL, int TEAM>
 cudaError_t launch_pts_one(const ProjParams<float> &p, const Tiling &t, cudaStream_t st)
 {
     static size_t granted = 0;  // per instantiation
-    size_t smem = t.smem;
-    if (WL && smem + fix_bytes(p.n_p, NF) <= kSmemCap) smem += fix_bytes(p.n_p, NF);
+    const int grid = (p.N + t.S - 1) / t.S;
+    // (teams of four: one CTA per SM by their registers)
+    const size_t smem = WL ? pts::pts_smem_with_fix(t.smem, t.smem_fix, TEAM < 4 && grid > sm_count()) : t.smem;
     cudaError_t e = reserve_smem(pts::pts_kernel<G, DIMS, NF, WL, TEAM>, smem, granted);
     if (e != cudaSuccess) return e;
-    const int grid = (p.N + t.S - 1) / t.S;
     return launch_pdl(pts::pts_kernel<G, DIMS, NF, WL, TEAM>, dim3(grid), dim3(t.threads), smem, st, p);
 }
 
@@ -150,16 +162,13 @@ cudaError_t launch_pts_batch_one(const ProjParams<float> *params, const int2 *it
 {
     static size_t granted = 0;
     auto kern = pts::pts_batch_kernel<G, DIMS, NF, WL>;
-    if (WL) smem = std::min(kSmemCap, smem + fix_bytes(160, NF));
     cudaError_t e = reserve_smem(kern, smem, granted);
     if (e != cudaSuccess) return e;
     constexpr int threads = 32 * pts::kMaxWarps;
     if (grid <= 0) {
-        int per_sm = 0, dev = 0, n_sm = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        int per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-        grid = std::max(1, per_sm) * n_sm;
+        grid = std::max(1, per_sm) * sm_count();
     }
     kern<<<std::min(grid, n_items), threads, smem, st>>>(params, items, n_items, counter);
     return cudaGetLastError();
@@ -180,6 +189,11 @@ cudaError_t launch_pts_batch_wl(const ProjParams<float> *params, const int2 *ite
 }
 
 }  // namespace
+
+size_t pts_batch_smem(size_t smem, size_t smem_fix, int n_items)
+{
+    return pts::pts_smem_with_fix(smem, smem_fix, n_items > sm_count());
+}
 
 // Persistent point-owner launch over (problem, first sample) items, G lanes per sample.
 cudaError_t launch_project_pts_batch(const ProjParams<float> *params, const int2 *items, int n_items, int *counter,

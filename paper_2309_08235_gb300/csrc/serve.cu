@@ -390,6 +390,7 @@ cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vecto
         GroupLaunch gl{std::get<0>(g.first), std::get<1>(g.first), g.second.front()->h.sh.nv, 0, std::get<2>(g.first),
                        g.second.front()->t.R, np, ni, 0, 0};
         std::vector<std::pair<double, int2>> its;
+        size_t smem_fix = 0;
         for (Slot *s : g.second) {
             const Shape &sh = s->h.sh;
             ProjParams<Real> p = proj_params<Real>(ctx, &s->h, s->t);
@@ -408,6 +409,7 @@ cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vecto
             p.c1_out = s->h.c1;
             gl.want_lambda |= p.want_lambda;
             gl.smem = std::max(gl.smem, s->t.smem);
+            smem_fix = std::max(smem_fix, s->t.smem_fix);
             const int idx = int(np - gl.first_param);
             pp[np++] = p;
             const double cost = double(sh.n_p) * (double(sh.n_obs) + 12.0);
@@ -419,6 +421,7 @@ cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vecto
         });
         for (auto &x : its) items[ni++] = x.second;
         gl.n_items = ni - gl.first_item;
+        if (gl.kind == 1 && gl.want_lambda) gl.smem = pts_batch_smem(gl.smem, smem_fix, int(gl.n_items));
         launches.push_back(gl);
     }
     // ---- selection / refit arguments, in the order of the parameters above
