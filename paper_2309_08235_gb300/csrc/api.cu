@@ -388,15 +388,17 @@ void fill_result(const Shape &sh, const double *host_out, const double *host_mu,
     res->best_index = int(host_out[sh.D + 3]);
 }
 
-// Point-owner tilings of one persistent launch from all its samples; returns the
-// lanes per sample they share.
-int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles)
+// Point-owner tilings of one persistent launch from all its samples, with G lanes
+// per sample (0: the lanes follow from the samples too); returns G.
+int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles, int G)
 {
     size_t total = 0;
     for (const Shape &sh : shapes) total += size_t(sh.N);
     const int m = int((total + ctx->n_sm - 1) / ctx->n_sm);
-    int G = 16;
-    for (const Shape &sh : shapes) G = std::max(G, pts_group(sh, m));
+    if (G == 0) {
+        G = 16;
+        for (const Shape &sh : shapes) G = std::max(G, pts_group(sh, m));
+    }
     for (size_t i = 0; i < shapes.size(); ++i) tiles[i] = pts_batch_tiling(shapes[i], G, m);
     return G;
 }

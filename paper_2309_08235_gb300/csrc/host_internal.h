@@ -101,8 +101,8 @@ Carve carve(const Shape &sh, bool fp32, int z_iters, bool proj_buffers);
 // Points h's buffers into `base` laid out as k.
 void carve_ptrs(priest_loaded *h, char *base, const Carve &k, bool fp32, int z_iters, bool proj_buffers);
 
-// Point-owner tilings of one persistent launch; returns the lanes per sample.
-int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles);
+// Point-owner tilings of one persistent launch of G lanes per sample (0: chosen here, returned).
+int pts_batch_tiles(const priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles, int G = 0);
 
 template <typename Real>
 ProjParams<Real> proj_params(const priest_ctx *ctx, const priest_loaded *h, const Tiling &t);

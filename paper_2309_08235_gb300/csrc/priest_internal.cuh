@@ -334,6 +334,7 @@ bool pts_supported(const Shape &sh);
 size_t pts_smem_bytes(const Shape &sh, int G, int warps, int C);  // C warps per sample
 int pts_group(const Shape &sh, int samples_per_sm);    // lanes per sample (16 or 32)
 Tiling pts_tiling(const Shape &sh, int G, int warps);  // 32 / G samples per warp; smem 0: does not fit
+int pts_serve_group(const Shape &sh);                  // the same for a served request: from its own shape alone
 int pts_team_size(const Shape &sh, int samples_per_sm);  // warps per sample of a team, 0: no team
 Tiling pts_team_tiling(const Shape &sh, int teams, int C);  // teams of C warps, a sample each
 Tiling pts_batch_tiling(const Shape &sh, int G, int samples_per_sm);  // item of the persistent launch

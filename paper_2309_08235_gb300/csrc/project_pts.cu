@@ -99,6 +99,14 @@ int pts_group(const Shape &sh, int samples_per_sm)
     return (sh.dims == 2 && sh.nf == 5 && samples_per_sm > 16 && sh.n_p <= 16 * pts::kMaxStrides) ? 16 : 32;
 }
 
+// A served request shares its launches with whatever else is there, so its lanes
+// per sample, on which its sums depend, are its own shape's.  The busy server's: bursts
+// of 32 / 64 uneven requests take 5.8 / 9.1 ms with 16 lanes, 6.4 / 10.5 with 32, 6.3 /
+// 9.4 when requests below 512 samples have 32 (two launches a step, each with its
+// tail); a request alone takes 0.44 / 0.55 ms (64 samples, 50 / 300 obstacles) against
+// 0.40 / 0.45.
+int pts_serve_group(const Shape &sh) { return pts_group(sh, 1 << 20); }
+
 // Item of the persistent launch: as many warps as leave room for two CTAs per
 // SM, but at least four.  A launch with few samples per SM spreads them over two
 // CTAs of each SM; one with many takes kSamplesPerWarp rounds per item.

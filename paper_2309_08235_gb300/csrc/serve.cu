@@ -301,17 +301,19 @@ cudaError_t Server::enqueue_step(std::vector<Slot *> &active, const std::vector<
 template <typename Real>
 cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vector<Slot *> &fresh, Stage &sg)
 {
-    // ---- groups of the projection launch: same dims, free-coefficient count
-    //      and projection kernel; the point-owner tilings of a group follow from
-    //      all its samples
-    std::map<std::tuple<int, int, int>, std::vector<Slot *>> groups;
-    for (Slot *s : active) groups[{s->h.sh.dims, s->h.sh.nf, s->t.kind}].push_back(s);
+    // ---- groups of the projection launch: same dims, free-coefficient count,
+    //      projection kernel and lanes per sample; the point-owner tilings of a
+    //      group follow from all its samples (they change no result: the sums
+    //      depend on the lanes per sample, which are the request's own)
+    std::map<std::tuple<int, int, int, int>, std::vector<Slot *>> groups;
+    for (Slot *s : active)
+        groups[{s->h.sh.dims, s->h.sh.nf, s->t.kind, s->t.kind == 1 ? pts_serve_group(s->h.sh) : 0}].push_back(s);
     for (auto &g : groups) {
         if (std::get<2>(g.first) != 1) continue;
         std::vector<Shape> shapes;
         for (Slot *s : g.second) shapes.push_back(s->h.sh);
         std::vector<Tiling> tiles(shapes.size());
-        pts_batch_tiles(ctx, shapes, tiles);
+        pts_batch_tiles(ctx, shapes, tiles, std::get<3>(g.first));
         for (size_t i = 0; i < tiles.size(); ++i) g.second[i]->t = tiles[i];
     }
     // ---- layout of the staging block

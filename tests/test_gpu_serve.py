@@ -131,6 +131,36 @@ def test_mix_equals_alone_fp32(P):
         assert abs(m["c_aug"] - a["c_aug"]) <= TOL_FP32 * max(1.0, a["c_aug"])
 
 
+def test_load_changes_no_bit_fp32(P):
+    """A request's result is bitwise the same alone and under a load that fills the
+    GPU (above 16 samples per SM, where a launch of many samples would take other
+    lanes per sample than one of few), over four CEM iterations, 2-D and 3-D."""
+    import torch
+
+    reqs = []
+    for k in range(14):
+        dims = 3 if k % 5 == 4 else 2
+        p = scene(dims=dims, n_obs=10 + 3 * k, n_dyn=k % 3, n_p=(40, 77, 100, 256)[k % 4], seed=80 + k)
+        p["seed"] = 3000 + k
+        reqs.append((p, W.cem_settings(200 + 24 * k, 60, 4, dims=2)))
+    total = sum(cem["n_samples"] for p, cem in reqs if p["dims"] == 2)
+    assert total > 16 * torch.cuda.get_device_properties(0).multi_processor_count
+
+    def serve(alone):
+        with P.Context(*reqs[0], precision=P.PRIEST_FP32) as ctx:
+            if alone:
+                return [ctx.wait(ctx.submit(p, cem)) for p, cem in reqs], ctx.serve_stats()
+            tickets = [ctx.submit(p, cem) for p, cem in reqs]
+            return [ctx.wait(t) for t in tickets], ctx.serve_stats()
+
+    (alone, st_a), (mix, st_m) = serve(True), serve(False)
+    assert st_a["max_active"] == 1 and st_m["max_active"] > 8
+    for a, m in zip(alone, mix):
+        assert a["status"] == 0 and m["status"] == 0 and a["best_index"] == m["best_index"]
+        for k in ("best", "mu", "r", "c1", "c_aug"):
+            np.testing.assert_array_equal(a[k], m[k])
+
+
 def test_budget_admission_defers_and_matches(P):
     """A budget that holds about two requests at once: the rest wait for
     memory, every result is produced, peak memory stays within the budget,
