@@ -1075,11 +1075,13 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
         return (__any_sync(kAll, e_p > tauP2) ? 1 : 0) | (__any_sync(kAll, e_a > tauA2) ? 2 : 0);
     };
     // the warp's part of the rebuild, for every sample it holds.  Lists that lasted only a few
-    // iterations are rebuilt with twice the margin, those of too many pairs with half of it
-    // (never beyond the margin that the grid's cells were filled for, in its header); rounding
-    // may take two fifths of a margin
+    // iterations are rebuilt with twice the margin, those of too many pairs with half of it,
+    // which it then keeps to (never beyond the margin that the grid's cells were filled for, in
+    // its header); rounding may take two fifths of a margin.  (A margin doubled again after it
+    // overflowed built two or three lists a rebuild: 14 moving circles, 574 samples, K = 75,
+    // 341 us a pass against 266; 45, 400 samples, K = 60, 625 against 379.)
     float reach = delta;
-    const float widest = hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta;
+    float widest = hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta;
     int built = -kShortLived;
     auto rebuild = [&](int need, int k) {
         const bool need_p = need & 1, need_a = need & 2;
@@ -1103,6 +1105,7 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
                                              reinterpret_cast<int *>(smem() + hdr(kXchAt) + team * kXch + kXchEnd));
                     if (trips >= 0 || reach < 0.3f * delta) break;
                     reach *= 0.5f;
+                    widest = fmaxf(reach, 0.25f * delta);
                 }
                 if (trips < 0) reach = delta;
                 // (no list: nothing is tested, so every stride's workspace rows too)
