@@ -578,8 +578,10 @@ template <typename Real>
 Tiling pick_tiling(priest_ctx *ctx, const Shape &sh, int N, ProjParams<Real> p, cudaStream_t st)
 {
     const Tiling model = choose_tiling<Real>(sh, N, ctx->n_sm);
-    // the point-owner kernel has one tiling per shape (its sizes come from the SM's limits)
+    // the point-owner kernel has one tiling per shape (its sizes come from the SM's limits), and a
+    // crowded problem's route must not start trials when its obstacles have moved
     if (!ctx->cfg.autotune || model.kind == 1) return model;
+    if (sizeof(Real) == 4 && pts_crowded(sh, (N + ctx->n_sm - 1) / ctx->n_sm)) return model;
     const std::vector<int> key = {int(sizeof(Real)), sh.dims, sh.nv, sh.nf, sh.n_p, sh.n_obs, sh.n_static,
                                   N, p.want_lambda, sh.use_bounds};
     load_tune_cache(ctx);
@@ -1229,8 +1231,8 @@ priest_status tune_batch(priest_ctx *ctx, int n, const std::vector<Shape> &shape
 }
 
 // Per-problem tilings of one persistent launch and the kernel they share:
-// the point-owner kernel when every problem's tiling uses it, the chunked one
-// otherwise (one kernel kind per launch).
+// the point-owner kernel when every problem's tiling uses it and not all are
+// crowded (pts_crowded), the chunked one otherwise (one kernel kind per launch).
 template <typename Real>
 priest_status batch_tiles(priest_ctx *ctx, const std::vector<Shape> &shapes, std::vector<Tiling> &tiles, int &kind,
                           int &R)
@@ -1241,6 +1243,22 @@ priest_status batch_tiles(priest_ctx *ctx, const std::vector<Shape> &shapes, std
     for (int i = 0; i < n; ++i) {
         tiles[i] = batch_tiling_for<Real>(ctx, shapes[i]);
         all_pts = all_pts && tiles[i].kind == 1;
+    }
+    if (all_pts && sizeof(Real) == 4) {
+        // crowded problems alone: the chunked kernel, where it holds them all
+        size_t total = 0;
+        for (const Shape &sh : shapes) total += size_t(sh.N);
+        const int m = int((total + ctx->n_sm - 1) / ctx->n_sm);
+        bool crowded = true;
+        std::vector<Tiling> chunked(n);
+        for (int i = 0; i < n && crowded; ++i) {
+            chunked[i] = batch_tiling<Real>(shapes[i], true);
+            crowded = pts_crowded(shapes[i], m) && chunked[i].smem > 0;
+        }
+        if (crowded) {
+            tiles = chunked;
+            all_pts = false;
+        }
     }
     for (int i = 0; i < n && !all_pts; ++i)
         if (tiles[i].kind == 1) {

@@ -335,6 +335,7 @@ size_t pts_smem_bytes(const Shape &sh, int G, int warps, int C);  // C warps per
 int pts_group(const Shape &sh, int samples_per_sm);    // lanes per sample (16 or 32)
 Tiling pts_tiling(const Shape &sh, int G, int warps);  // 32 / G samples per warp; smem 0: does not fit
 int pts_serve_group(const Shape &sh);                  // the same for a served request: from its own shape alone
+bool pts_crowded(const Shape &sh, int samples_per_sm);  // the chunked kernel projects it faster
 int pts_team_size(const Shape &sh, int samples_per_sm);  // warps per sample of a team, 0: no team
 Tiling pts_team_tiling(const Shape &sh, int teams, int C);  // teams of C warps, a sample each
 Tiling pts_batch_tiling(const Shape &sh, int G, int samples_per_sm);  // item of the persistent launch
@@ -460,7 +461,7 @@ std::vector<Tiling> tiling_candidates(const Shape &sh, int n_samples, int n_sm);
 // variant's CTA size, warp groups of two (2-D FP32) or one warp, chunk count
 // from the cost model.  smem == 0 signals a problem too large for one CTA.
 template <typename Real>
-Tiling batch_tiling(const Shape &sh);
+Tiling batch_tiling(const Shape &sh, bool chunked = false);  // chunked: never the point-owner kernel
 template <typename Real>
 std::vector<Tiling> batch_candidates(const Shape &sh);
 

@@ -2,6 +2,7 @@
 // (project_kernel.cuh): a cost model for the default tiling and the list of
 // compiled (points per item, CTA size) variants the autotuner times.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <string>
 #include <vector>
@@ -69,6 +70,38 @@ bool pts_allowed()
     return allowed;
 }
 
+// Where the chunked kernel projects a shape that the point-owner kernel covers: in
+// 2-D, among many obstacles that mostly move (no grid), most pairs are active, and the
+// chunked kernel's sums per time stamp are cheaper than the pairs' own.  How many are
+// active follows from the share of the obstacles' box that their discs fill (crowd)
+// and, at the same share, from how near the straight line's mean speed is to the
+// bound: a sample with no speed to spare cannot leave the obstacles it is in.
+// Point-owner / chunked, us a pass (K = 50 to 92; 110, 1,000 and 2,000 samples):
+//   mean speed above the bound, share 0.19:  143 / 129, 210 / 187, 247 / 341
+//                               share 0.27:  164 / 136, 239 / 195, 271 / 364
+//                               share 0.43:  221 / 165, 341 / 280, 386 / 605
+//                               share 0.69:  270 / 154, 420 / 272, 472 / 606
+//   0.55 of the bound,          share 0.69:  210 / 209, 261 / 425, 286 / 959
+//                               share 1.34:  257 / 258, 440 / 652, 664 / 1622
+//                               share 2.66:  524 / 357, 803 / 1051, 5645 / 2819
+//   seven columns, above,       share 0.32:  177 / 241, 271 / 331, 405 / 719
+//                               share 0.55:  273 / 262, 394 / 374, 600 / 872
+//   share 0.42, by the mean speed over the bound, 110 and 400 samples: 1.0 189 / 166 and
+//   292 / 212, 0.89 177 / 167 and 279 / 213, 0.8 167 / 167 and 264 / 213, 0.67 145 / 165 and
+//   219 / 213 (share 0.27: 0.89 147 / 146 and 230 / 187, 0.67 130 / 146 and 175 / 192)
+// (circles on a corridor and, at 0.55 of the bound, crossing traffic).  3-D: the point-owner
+// kernel is faster at every share (33 to 200 spheres: 127 to 386 against 186 to 1,021).
+// The route depends on the obstacles' values, so it takes the model's tiling: trial
+// launches would stall a replanner in the middle of its run, or break its capture.
+bool pts_crowded(const Shape &sh, int samples_per_sm)
+{
+    if (!pts_supported(sh) || sh.dims != 2 || sh.n_static >= kGridMinStatic || sh.n_obs < 12) return false;
+    double d2 = 0.0;
+    for (int ax = 0; ax < sh.dims; ++ax) d2 += (sh.bf[ax][0] - sh.b0[ax][0]) * (sh.bf[ax][0] - sh.b0[ax][0]);
+    const bool hurried = std::sqrt(d2) > 0.85 * sh.vmax * sh.horizon;
+    return sh.crowd >= (!hurried ? 2.0 : sh.nf == 5 && samples_per_sm <= 8 ? 0.25 : 1.0);
+}
+
 // Default tiling: the point-owner kernel for the shapes it covers; otherwise the
 // largest compiled variant, the largest warp group that
 // fits the CTA, and the obstacle chunk count that gives each group's threads
@@ -76,14 +109,11 @@ bool pts_allowed()
 template <typename Real>
 Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
 {
-    // Where many obstacles, almost all moving (no grid), fill half of their box with their discs,
-    // most pairs are active and the sums per time stamp of the chunked kernel are cheaper than
-    // the pairs' own (41 moving circles on a corridor, share 0.59, 755 samples: 123 against 216
-    // us; 22, share 0.35, the lists are faster; batched launches keep one kernel for all problems).
-    const bool crowded = sh.n_static < kGridMinStatic && sh.n_obs >= 32 && sh.crowd >= 0.5;
+    const int m = std::max(1, (n_samples + n_sm - 1) / n_sm);
+    const bool crowded = sizeof(Real) == 4 && pts_crowded(sh, m);
     if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed() && !crowded) {
         // an SM's share of the samples in as few CTAs of equal size as hold them
-        const int m = std::max(1, (n_samples + n_sm - 1) / n_sm), G = pts_group(sh, m);
+        const int G = pts_group(sh, m);
         // few samples per SM: a team of warps for each (pts_team_size)
         if (const int C = pts_team_size(sh, m)) {
             const int fit = 8 / C, n = (m + fit - 1) / fit;
@@ -95,7 +125,7 @@ Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
         if (p.smem > 0) return p;
     }
     Tiling t;
-    t.R = sizeof(Real) == 8 ? 4 : 5;
+    t.R = sizeof(Real) == 8 || crowded ? 4 : 5;  // (crowded: 141 against 174 us with 5, 33 circles, 110 samples)
     t.threads = sizeof(Real) == 8 ? 256 : 512;
     const int S0 = std::max(1, (n_samples + n_sm - 1) / n_sm);
     t.ws = 1;
@@ -146,9 +176,9 @@ std::vector<Tiling> tiling_candidates(const Shape &sh, int n_samples, int n_sm)
 }
 
 template <typename Real>
-Tiling batch_tiling(const Shape &sh)
+Tiling batch_tiling(const Shape &sh, bool chunked)
 {
-    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed()) {
+    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed() && !chunked) {
         const Tiling p = pts_batch_tiling(sh, pts_group(sh, 1 << 20), 1 << 20);
         if (p.smem > 0) return p;
     }
@@ -257,8 +287,8 @@ template Tiling choose_tiling<float>(const Shape &, int, int);
 template Tiling choose_tiling<double>(const Shape &, int, int);
 template std::vector<Tiling> tiling_candidates<float>(const Shape &, int, int);
 template std::vector<Tiling> tiling_candidates<double>(const Shape &, int, int);
-template Tiling batch_tiling<float>(const Shape &);
-template Tiling batch_tiling<double>(const Shape &);
+template Tiling batch_tiling<float>(const Shape &, bool);
+template Tiling batch_tiling<double>(const Shape &, bool);
 template std::vector<Tiling> batch_candidates<float>(const Shape &);
 template std::vector<Tiling> batch_candidates<double>(const Shape &);
 template cudaError_t launch_project<float>(const ProjParams<float> &, const Tiling &, cudaStream_t);

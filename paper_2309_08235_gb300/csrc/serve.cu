@@ -247,6 +247,10 @@ bool Server::admit(std::unique_lock<std::mutex> &, std::vector<Slot *> &active, 
         s->h.bytes = k.total;
         s->status = reinterpret_cast<int *>(s->h.out + s->h.sh.D + 4);
         s->t = fp32 ? batch_tiling<float>(s->h.sh) : batch_tiling<double>(s->h.sh);
+        if (fp32 && pts_crowded(s->h.sh, 1 << 20)) {
+            const Tiling c = batch_tiling<float>(s->h.sh, true);
+            if (c.smem > 0) s->t = c;
+        }
         if (rb) {
             s->robot = rb;
             rb->busy = true;
