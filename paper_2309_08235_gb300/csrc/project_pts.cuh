@@ -573,14 +573,16 @@ template <int G, int DIMS, int NF>
 __device__ __forceinline__ Rounding row_rounding(const float2 (&c)[NF][DIMS], float vmax, float amax)
 {
     static_assert(NF == 5 || NF == 7, "kappa");
-    float most = 0.f, extent = smem()[kExtent];
+    float most = 0.f, sum = 0.f, extent = smem()[kExtent];
 #pragma unroll
     for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int ax = 0; ax < DIMS; ++ax) {
             most = fmaxf(most, fabsf(c[f][ax].x));
+            sum += fabsf(c[f][ax].x);
             extent = fmaxf(extent, fabsf(c[f][ax].x - smem()[kOrigin + ax]));
         }
+    if (!(sum <= FLT_MAX)) most = INFINITY;  // a NaN, which the maxima drop, has no margin
     if (G == 16) {
         most = fmaxf(most, __shfl_xor_sync(kAll, most, 16));
         extent = fmaxf(extent, __shfl_xor_sync(kAll, extent, 16));
@@ -1068,8 +1070,9 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
 #pragma unroll
                 for (int ax = 0; ax < DIMS; ++ax) e[ax] = ffma2(node[f], m[f][ax], e[ax]);
             const float2 n = norm2<DIMS>(e);
-            e_p = fmaxf(e_p, n.x);
-            e_a = fmaxf(e_a, n.y);
+            // (a NaN or an overflow is beyond every finite threshold)
+            e_p = fmaxf(e_p, fminf(n.x, FLT_MAX));
+            e_a = fmaxf(e_a, fminf(n.y, FLT_MAX));
         }
         if (!__any_sync(kAll, e_p > tauP2 || e_a > tauA2)) return 0;
         return (__any_sync(kAll, e_p > tauP2) ? 1 : 0) | (__any_sync(kAll, e_a > tauA2) ? 2 : 0);

@@ -1,0 +1,37 @@
+"""The FP32 point-owner projection at the limits of its inputs and lists, in every form
+(teams of four and of two warps per sample, one warp, two samples per warp): bitwise the
+results of screening every pair in every iteration, and the FP64 oracle's where these
+are finite."""
+import numpy as np
+import pytest
+
+from gpu_common import TOL_FP32, rel_err, samples, scale_of, scene
+from test_gpu_pts_edges import P, PER_SM, project, sm_count  # noqa: F401
+from test_gpu_pts_frames import same
+
+pytestmark = pytest.mark.gpu
+
+FORMS = pytest.mark.parametrize("form", list(PER_SM))
+SHAPES = pytest.mark.parametrize("dims,mask", [(2, 7), (3, 7), (2, 1)])
+
+
+@SHAPES
+@FORMS
+@pytest.mark.parametrize("bounds", [False, True])
+def test_coefficient_turns_nan(P, oracle, bounds, form, dims, mask):  # noqa: F811
+    """A multiplier beyond FP32's range makes one axis infinite, then NaN, after the lists
+    were built: what that does to the other axes is the same with lists and without,
+    and other samples are untouched."""
+    p = scene(dims=dims, n_obs=12, n_dyn=2, n_p=60, mask=mask, bounds=bounds, vmax=30.0, amax=60.0)
+    n = PER_SM[form] * sm_count() - 3
+    xi = samples(oracle, p, n, seed=3)
+    lam0 = np.zeros_like(xi)
+    good = project(P, p, xi, 8, lam0, "1")
+    odd = lam0.copy()
+    odd[::5, 5] = 1e300
+    got = project(P, p, xi, 8, odd, "1")
+    same(got, project(P, p, xi, 8, odd, "0"))
+    assert np.isnan(got[0][::5]).any(axis=1).all()
+    rest = np.arange(n) % 5 != 0
+    for x, y in zip(got, good):
+        np.testing.assert_array_equal(x[rest], y[rest])
