@@ -29,13 +29,13 @@ constexpr int kXchFlag = 3 * 32, kXchBuf = kXchFlag + 8, kXchEnd = 2 * kXchBuf, 
 //   tv    [np]                time stamps
 //   node  [32 / G][nfn][32][4]  node rows {P, Pdd} of two columns a time (nfn = (nf + 1) / 2)
 //   obs   [n_obs][4]          2-D {1/a, -o_x/a, -o_y/a, a}, 3-D {1/a, -o_x/a, -o_y/a, -o_z/b}
-//   obq   [n_obs][4]          3-D {1/b, a, b, max(1/a, 1/b)}
+//   obq   [n_obs][4]          3-D {kUnit/b, a, b, max(1/a, 1/b)}
 //   mov   [n_moving][4]       {-v_x/a, -v_y/a[, -v_z/b]}
 //   grid  [gl.smem]           the static-obstacle grid of the tables
 //   per warp, for each of its 32 / G samples:
 //     c [nf][4 | 8]           coefficients, each twice: {x, x, y, y[, z, z, -, -]}
 //     stage [4 G][4]          active pairs on their way to a lane: {r (dims), t}
-//     list [kPairs][4]        2-D {1/a, -o_x(t)/a, -o_y(t)/a, a}, 3-D {1/a, -o_x(t)/a, -o_y(t)/a, -o_z(t)/b}
+//     list [kPairs][4]        kUnit {1/a, -o_x(t)/a, -o_y(t)/a} and 2-D a, 3-D -kUnit o_z(t)/b
 //     tj [kPairs]             (ints) time stamp | obstacle << 16
 //     moved [nf][dims][2]     coefficients since the rebuild of the {pair, rate} lists
 //   xch   [teams][kXch]       what a team's warps tell one another

@@ -35,3 +35,25 @@ def test_coefficient_turns_nan(P, oracle, bounds, form, dims, mask):  # noqa: F8
     rest = np.arange(n) % 5 != 0
     for x, y in zip(got, good):
         np.testing.assert_array_equal(x[rest], y[rest])
+
+
+@pytest.mark.parametrize("dims", [2, 3])
+@FORMS
+def test_next_to_the_centre(P, oracle, form, dims):  # noqa: F811
+    """A robot at rest within 1e-18 of an obstacle's centre: squared offsets are denormal
+    in FP32, the push is the semi-axis all the same.  One iteration; a denormal square of
+    1e-40 holds five digits, those below 1e-43 belong to the time stamps next to the
+    ends, whose rows weigh less than 1e-3: 5e-3 of the largest push allowed."""
+    p = scene(dims=dims, n_obs=1, n_dyn=0, n_p=60, radius=(1.0, 1.0), vmax=1e6, amax=1e6)
+    p = dict(p, center=np.zeros((1, dims)), b0=np.zeros((dims, 3)), bf=np.zeros((dims, 3)))
+    n = PER_SM[form] * sm_count() - 3
+    rng = np.random.default_rng(5)
+    xi = np.zeros((n, dims, 11))
+    xi[:, :, 3:8] = 1e-19 * (rng.choice([-1.0, 1.0], (n, dims, 1)) + 0.1 * rng.normal(size=(n, dims, 5)))
+    xi = xi.reshape(n, -1)
+    got = project(P, p, xi, 1, None, "1")
+    same(got, project(P, p, xi, 1, None, "0"))
+    idx = np.r_[0:n:max(1, n // 20), n - 1]
+    xb_o, _ = oracle.project(p, xi[idx], 1)
+    assert np.abs(xb_o).max() > 0.01
+    assert np.abs(got[0][idx] - xb_o).max() < 5e-3 * np.abs(xb_o).max()
