@@ -1,11 +1,14 @@
 """The FP32 point-owner projection at the limits of its inputs and lists, in every form
 (teams of four and of two warps per sample, one warp, two samples per warp): bitwise the
-results of screening every pair in every iteration, and the FP64 oracle's where these
-are finite."""
+results of screening every pair in every iteration."""
+import os
+from math import comb
+
 import numpy as np
 import pytest
 
-from gpu_common import TOL_FP32, rel_err, samples, scale_of, scene
+from gpu_common import samples, scene
+from paper_2309_08235_gb300 import workloads as W
 from test_gpu_pts_edges import P, PER_SM, project, sm_count  # noqa: F401
 from test_gpu_pts_frames import same
 
@@ -57,3 +60,56 @@ def test_next_to_the_centre(P, oracle, form, dims):  # noqa: F811
     xb_o, _ = oracle.project(p, xi[idx], 1)
     assert np.abs(xb_o).max() > 0.01
     assert np.abs(got[0][idx] - xb_o).max() < 5e-3 * np.abs(xb_o).max()
+
+
+def near_pairs(p, xb, grow):
+    """Per sample, the (time stamp, obstacle) pairs within `grow` semi-axes."""
+    dims, n_p = p["dims"], p["n_p"]
+    tau = np.arange(n_p) / (n_p - 1)
+    B = np.stack([comb(10, j) * tau ** j * (1 - tau) ** (10 - j) for j in range(11)], 1)
+    x = np.einsum("tj,naj->nta", B, np.asarray(xb).reshape(len(xb), dims, 11))
+    o = np.asarray(p["center"]) + (tau * p["horizon"])[:, None, None] * np.asarray(p["vel"])
+    s = np.asarray(p["semi"])[:, [0, 0, 1][:dims]]
+    d = (x[:, :, None, :] - o) / s
+    return np.count_nonzero((d * d).sum(3) < grow * grow, axis=(1, 2))
+
+
+def crowd(dims, mask, kind):
+    if kind == "pile":  # every time stamp inside several obstacles, to the end
+        return scene(dims=dims, n_obs=40, n_dyn=5, n_p=70, mask=mask, radius=(3.0, 5.0))
+    # forty obstacles on one spot of the straight line, which the samples leave
+    p = scene(dims=dims, n_obs=40, n_dyn=0, n_p=70, mask=mask)
+    mid = 0.5 * (np.asarray(p["b0"])[:, 0] + np.asarray(p["bf"])[:, 0])
+    return dict(p, center=np.tile(mid, (40, 1)), semi=np.full((40, 2), 1.4), vel=np.zeros((40, dims)))
+
+
+K_LONG = 48  # three times the iterations after which a list that overflowed is tried again
+
+
+@pytest.mark.parametrize("kind", ["pile", "cleared"])
+@SHAPES
+@FORMS
+def test_lists_overflow_and_return(P, oracle, kind, form, dims, mask):  # noqa: F811
+    """More pairs than a list holds (256), for good or until the samples have moved
+    away, over several of the tries at a new list: bitwise as without lists."""
+    p = crowd(dims, mask, kind)
+    n = PER_SM[form] * sm_count() - 3
+    xi = samples(oracle, p, n, seed=3, std=0.3)
+    idx = np.r_[0:n:max(1, n // 9), n - 1]
+    assert (near_pairs(p, oracle.project_eq(p, xi[idx]), 1.0) > 256).all()
+    if kind == "cleared":
+        assert (near_pairs(p, oracle.project(p, xi[idx], 16)[0], 2.5) <= 256).all()
+    same(project(P, p, xi, K_LONG, np.zeros_like(xi), "1"), project(P, p, xi, K_LONG, np.zeros_like(xi), "0"))
+
+
+def test_default_margin_changes_no_bit(P, oracle):  # noqa: F811
+    """The margin set by the obstacles' density against a fixed one."""
+    p = W.scene_clutter_2d(seed=3, n_static=90, n_dyn=10, n_p=100)
+    xi = oracle.default_mean(p) + 2.0 * W.normals(77, (300, 22))
+    lam0 = np.random.default_rng(8).normal(0.0, 0.1, xi.shape)
+    got = project(P, p, xi, 40, lam0, "1")
+    os.environ["PRIEST_LIST_MARGIN"] = "0.75"
+    try:
+        same(got, project(P, p, xi, 40, lam0, "1"))
+    finally:
+        os.environ.pop("PRIEST_LIST_MARGIN")
