@@ -109,25 +109,28 @@ bool pts_crowded(const Shape &sh, int samples_per_sm)
 template <typename Real>
 Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
 {
-    const int m = std::max(1, (n_samples + n_sm - 1) / n_sm);
+    const int m = std::max(1, (n_samples + n_sm - 1) / n_sm);  // an SM's share of the samples
     const bool crowded = sizeof(Real) == 4 && pts_crowded(sh, m);
-    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed() && !crowded) {
-        // an SM's share of the samples in as few CTAs of equal size as hold them
-        const int G = pts_group(sh, m);
-        // few samples per SM: a team of warps for each (pts_team_size)
+    Tiling own;
+    own.smem = 0;
+    if (sizeof(Real) == 4 && pts_supported(sh) && pts_allowed()) {
+        // the share in as few CTAs of equal size as hold it; few samples per SM: a team of warps
+        // for each (pts_team_size)
         if (const int C = pts_team_size(sh, m)) {
             const int fit = 8 / C, n = (m + fit - 1) / fit;
-            const Tiling q = pts_team_tiling(sh, (m + n - 1) / n, C);
-            if (q.smem > 0 && size_t(n) * (q.smem + 1024) <= size_t(228) * 1024) return q;
+            own = pts_team_tiling(sh, (m + n - 1) / n, C);
+            if (size_t(n) * (own.smem + 1024) > size_t(228) * 1024) own.smem = 0;
         }
-        const int w = (m * G + 31) / 32, ctas = (w + 7) / 8;
-        const Tiling p = pts_tiling(sh, G, (w + ctas - 1) / ctas);
-        if (p.smem > 0) return p;
+        if (own.smem == 0) {
+            const int G = pts_group(sh, m), w = (m * G + 31) / 32, ctas = (w + 7) / 8;
+            own = pts_tiling(sh, G, (w + ctas - 1) / ctas);
+        }
+        if (own.smem > 0 && !crowded) return own;
     }
     Tiling t;
     t.R = sizeof(Real) == 8 || crowded ? 4 : 5;  // (crowded: 141 against 174 us with 5, 33 circles, 110 samples)
     t.threads = sizeof(Real) == 8 ? 256 : 512;
-    const int S0 = std::max(1, (n_samples + n_sm - 1) / n_sm);
+    const int S0 = m;
     t.ws = 1;
     while (t.ws < 8 && S0 * 32 * (2 * t.ws) <= t.threads && S0 <= 15) t.ws *= 2;
     int S = samples_per_cta(n_samples, n_sm, t.threads, t.ws);
@@ -139,7 +142,8 @@ Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
     t.S = S;
     t.C = C;
     t.smem = project_smem_bytes<Real>(sh, S, C);
-    return t;
+    // (the chunked kernel stages whole tables: it holds fewer obstacles and time stamps)
+    return t.smem > kSmemCap && own.smem > 0 ? own : t;
 }
 
 // Candidates for the autotuner: every compiled variant for the dimension,

@@ -58,6 +58,7 @@ CASES = {
     "seven": (lambda: traffic(20, 0.9, mask=1), 300, False),
     "seven_full": (lambda: traffic(20, 1.1, mask=1), 300, True),
     "three_d": (lambda: traffic(40, 2.5, dims=3), 300, False),
+    "too_large": (lambda: traffic(2048, 3.0, n_p=512), 6, False),  # beyond the chunked kernel's tables
 }
 
 
