@@ -1192,7 +1192,7 @@ priest_status tune_batch(priest_ctx *ctx, int n, const std::vector<Shape> &shape
                 e = cudaMemsetAsync(cnt, 0, sizeof(int), st);
                 if (e == cudaSuccess) e = cudaEventRecord(e0, st);
                 if (e == cudaSuccess)
-                    e = launch_project_batch<Real>(dp + k, di, int(it.size()), cnt, sh.dims, t.R, 0, sh.nf, sh.nv, 0,
+                    e = launch_project_batch<Real>(dp + k, di, int(it.size()), cnt, sh.dims, t.R, sh.nf, sh.nv, 0,
                                                    t.smem, 0, st, t.kind);
                 ctx->launches++;
                 if (e == cudaSuccess) e = cudaEventRecord(e1, st);
@@ -1513,7 +1513,7 @@ priest_status batch_enqueue(priest_ctx *ctx, BatchPlan *b, bool shape_ready, cud
         }
         if (e == cudaSuccess)
             e = launch_project_batch<Real>(params + size_t(l) * b->n, b->items_dev, b->n_items, b->counters_dev + l,
-                                           b->dims, b->R, 0, b->nf, b->nv, 0, b->smem_proj, 0, st, b->kind);
+                                           b->dims, b->R, b->nf, b->nv, 0, b->smem_proj, 0, st, b->kind);
         if (mark && e == cudaSuccess) e = cudaEventRecordWithFlags(b->ev[2 * l + 1], st, cudaEventRecordExternal);
         if (ev.first) {
             cudaEventRecord(ev.second, st);
@@ -1769,7 +1769,7 @@ priest_status project_batch(priest_ctx *ctx, int n, priest_loaded *const *probs,
     const Shape &s0 = shapes[0];
     cudaError_t e = launch_project_batch<Real>(reinterpret_cast<const ProjParams<Real> *>(db + o_par),
                                                reinterpret_cast<const int2 *>(db + o_it), int(items.size()),
-                                               reinterpret_cast<int *>(db), s0.dims, R, 0, s0.nf, s0.nv, want_lambda,
+                                               reinterpret_cast<int *>(db), s0.dims, R, s0.nf, s0.nv, want_lambda,
                                                smem, 0, st, kind);
     ctx->launches++;
     ctx->last_kind = kind;

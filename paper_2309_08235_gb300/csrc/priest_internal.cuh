@@ -437,7 +437,7 @@ size_t refit_smem_bytes(int D, int n_elite);
 // selects the chunked (0) or point-owner FP32 (1) kernel.
 template <typename Real>
 cudaError_t launch_project_batch(const ProjParams<Real> *params_dev, const int2 *items_dev, int n_items,
-                                 int *counter_dev, int dims, int R, int threads, int nf, int nv, int want_lambda,
+                                 int *counter_dev, int dims, int R, int nf, int nv, int want_lambda,
                                  size_t smem, int grid, cudaStream_t st, int kind = 0);
 
 

@@ -255,11 +255,9 @@ cudaError_t launch_project(const ProjParams<Real> &p, const Tiling &t, cudaStrea
 // (R = 5, 512 threads), 3-D (R = 5, 512 threads), FP64 (R = 4, 256 threads).
 template <typename Real>
 cudaError_t launch_project_batch(const ProjParams<Real> *params_dev, const int2 *items_dev, int n_items,
-                                 int *counter_dev, int dims, int R, int threads, int nf, int nv, int want_lambda,
+                                 int *counter_dev, int dims, [[maybe_unused]] int R, int nf, int nv, int want_lambda,
                                  size_t smem, int grid, cudaStream_t st, int kind)
 {
-    (void)threads;
-    (void)R;
     if (n_items <= 0) return cudaSuccess;
     if constexpr (sizeof(Real) == 4) {
         if (kind == 1)
@@ -282,9 +280,9 @@ cudaError_t launch_project_batch(const ProjParams<Real> *params_dev, const int2 
 }
 
 template cudaError_t launch_project_batch<float>(const ProjParams<float> *, const int2 *, int, int *, int, int, int,
-                                                 int, int, int, size_t, int, cudaStream_t, int);
+                                                 int, int, size_t, int, cudaStream_t, int);
 template cudaError_t launch_project_batch<double>(const ProjParams<double> *, const int2 *, int, int *, int, int,
-                                                  int, int, int, int, size_t, int, cudaStream_t, int);
+                                                  int, int, int, size_t, int, cudaStream_t, int);
 template size_t project_smem_bytes<float>(const Shape &, int, int);
 template size_t project_smem_bytes<double>(const Shape &, int, int);
 template Tiling choose_tiling<float>(const Shape &, int, int);

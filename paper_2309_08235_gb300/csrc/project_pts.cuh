@@ -1610,16 +1610,12 @@ __global__ void __launch_bounds__(32 * kMaxWarps, TEAM == 4 ? 1 : 2) pts_kernel(
     pts_body<G, DIMS, NF, WL, TEAM>(p, s0, min(p.S, p.N - s0), p.WS);
 }
 
-// CTAs of the persistent form per SM that its registers allow.
-template <int DIMS, int NF>
-constexpr int pts_batch_ctas_per_sm() { return 2; }
-
 // Persistent form over many problems: CTAs take (problem, first sample)
 // items (p.S samples by p.WS warps) through an atomic counter until none is
 // left; the item's parameters are staged in shared memory.  *next must be zero
 // at launch.
 template <int G, int DIMS, int NF, bool WL>
-__global__ void __launch_bounds__(32 * kMaxWarps, pts_batch_ctas_per_sm<DIMS, NF>())
+__global__ void __launch_bounds__(32 * kMaxWarps, 2)
     pts_batch_kernel(const ProjParams<float> *params, const int2 *items, int n_items, int *next)
 {
     __shared__ int s_item;

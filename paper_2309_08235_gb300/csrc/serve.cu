@@ -472,7 +472,7 @@ cudaError_t Server::enqueue_step_t(std::vector<Slot *> &active, const std::vecto
     for (size_t gi = 0; gi < launches.size(); ++gi) {
         const GroupLaunch &gl = launches[gi];
         e = launch_project_batch<Real>(ppd + gl.first_param, itd + gl.first_item, int(gl.n_items), cnt + gi, gl.dims,
-                                       gl.R, 0, gl.nf, gl.nv, gl.want_lambda, gl.smem, 0, st, gl.kind);
+                                       gl.R, gl.nf, gl.nv, gl.want_lambda, gl.smem, 0, st, gl.kind);
         ctx->launches++;
         if (e != cudaSuccess) return e;
     }
