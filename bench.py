@@ -24,6 +24,7 @@ the same workload on this host's cores.
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
 import statistics
@@ -190,6 +191,22 @@ def stored_profile(key):
         if ln.startswith(key + ":"):
             return float(ln.split(":", 1)[1].split()[0])
     return None
+
+
+def kernel_digest():
+    """Digest of the point-owner kernel's source without comments and spacing: the
+    stored ncu figures are printed only for the kernel they were captured from."""
+    h = hashlib.sha256()
+    for name in ("project_pts.cuh", "pts_layout.cuh"):
+        with open(os.path.join(ROOT, "paper_2309_08235_gb300", "csrc", name)) as f:
+            h.update("".join("".join(ln.split("//", 1)[0].split()) for ln in f).encode())
+    return h.hexdigest()[:16]
+
+
+def profile_current():
+    """Whether profiles/traffic.txt was captured from the kernel as it is."""
+    path = os.path.join(ROOT, "profiles", "traffic.txt")
+    return os.path.exists(path) and any(ln.split() == ["pts_kernel_source:", kernel_digest()] for ln in open(path))
 
 
 SCREEN_NOTE = ("achieved counts the scope table's per-unit work: the direct polar test of every (point, obstacle) pair "
@@ -401,7 +418,7 @@ def measure_single(args, name, steps, warmup, precision="fp32", plain_steps=0, e
     kname = {0: "project_kernel (FP32 chunked projection)", 1: "pts_kernel (FP32 point-owner projection)",
              2: "project_tc_kernel (tcgen05 pair tests)"}.get(kind, "projection kernel")
     # the committed ncu figures of this workload's point-owner launch, where one was captured
-    prof = {"clutter2d": "pts_kernel", "ellipsoid3d": "pts_kernel_3d"}.get(name) if kind == 1 else None
+    prof = {"clutter2d": "pts_kernel", "ellipsoid3d": "pts_kernel_3d"}.get(name) if kind == 1 and profile_current() else None
     traffic = stored_profile(f"{prof}_bytes_per_launch") if prof else None
     traffic = None if traffic is None else int(traffic)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
@@ -589,7 +606,7 @@ def run_batched(args):
     achieved = flops_launch / (avg_proj_ms / 1e3) / 1e12
     kname = {0: "project_batch_kernel (FP32 chunked, persistent)",
              1: "pts_batch_kernel (FP32 point-owner, persistent)"}.get(kind, "batched projection kernel")
-    traffic = stored_profile("pts_batch_kernel_bytes_per_launch") if kind == 1 else None
+    traffic = stored_profile("pts_batch_kernel_bytes_per_launch") if kind == 1 and profile_current() else None
     traffic = None if traffic is None else int(traffic)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": traffic, "kernel": kname, "avg_launch_ms": avg_proj_ms, "launches": n_proj_launch,
@@ -602,7 +619,8 @@ def run_batched(args):
                                  "(profiles/traffic.txt), not measured in this run") if traffic else None}
     if kind == 1:
         roofline["note"] = SCREEN_NOTE
-        roofline["executed"] = executed("pts_batch_kernel")
+        if profile_current():
+            roofline["executed"] = executed("pts_batch_kernel")
     if clocks.get("sm_mhz"):
         roofline["frac_at_median_clock"] = achieved / fp32_peak_tflops(n_sm, clocks["sm_mhz"])
 
