@@ -97,7 +97,9 @@ typedef struct {
                               requests into (0 = 2 GiB); its small per-step staging is extra */
     int autotune;          /* 1: time candidate tilings of the projection kernel on the first
                               call of each problem shape and keep the fastest (the first call
-                              then blocks for the trials); 0: cost-model tiling */
+                              then blocks for the trials); 0: cost-model tiling.  FP32 problems
+                              of the point-owner kernel (degree 10 with 5 free coefficients per
+                              axis, or 7 in 2-D) have one tiling and no trials */
     int serve_slots;       /* most requests the serving loop keeps on the device at once
                               (0 = as many as the budget holds) */
 } priest_config;
@@ -204,7 +206,8 @@ priest_status priest_plan_multi(priest_ctx *ctx, const priest_problem *prob, int
  * allocated once at the first submit) and cfg.serve_slots, and advances every
  * admitted request by one CEM iteration per step, all of them in shared
  * launches: one persistent projection launch per (dims, free-coefficient
- * count) group, one selection and one refit launch.  Requests submitted while
+ * count) group, one selection and one refit launch.  A request's result does
+ * not depend on what else is being served, to the last bit.  Requests submitted while
  * others are on the device join at the next step; memory of finished
  * requests returns to the budget at once.  The standard-normal draws come
  * from prob->seed through the same stream as priest_rng_normal, computed on
@@ -430,7 +433,7 @@ priest_status priest_profile_read(priest_ctx *ctx, int64_t *launches, double *ms
  * Kernels: those of priest_project with the cost-model tiling (no timing of
  * candidate tilings): in FP32 the point-owner kernel for the degree-10
  * shapes it covers (five free coefficients, or seven in 2-D), the chunked
- * kernel otherwise; obstacles are reordered static-first on the device, as
+ * kernel otherwise and in crowded 2-D scenes; obstacles are reordered static-first on the device, as
  * priest_project orders them.
  * Scratch: one fixed 1 MiB device array inside the library, held by every
  * device that loads it until the process exits; every call shares it and it

@@ -101,10 +101,11 @@ int pts_group(const Shape &sh, int samples_per_sm)
 
 // A served request shares its launches with whatever else is there, so its lanes
 // per sample, on which its sums depend, are its own shape's.  The busy server's: bursts
-// of 32 / 64 uneven requests take 5.8 / 9.1 ms with 16 lanes, 6.4 / 10.5 with 32, 6.3 /
-// 9.4 when requests below 512 samples have 32 (two launches a step, each with its
-// tail); a request alone takes 0.44 / 0.55 ms (64 samples, 50 / 300 obstacles) against
-// 0.40 / 0.45.
+// of 8 / 32 / 64 uneven requests take 2.1 / 5.8 / 9.1 ms with 16 lanes, 2.3 / 6.4 / 10.5
+// with 32, 2.5 / 6.3 / 9.4 when requests below 512 samples have 32 (two launches a
+// step, each with its tail).  The price is a request alone: 0.44 / 0.55 ms (64 samples, 50
+// / 300 obstacles) against 0.40 / 0.45 with 32 lanes; arrivals at 500 / 2,000 a second see
+// a median of 0.71 / 1.47 ms against 0.61 / 1.33 (p99 1.84 / 3.65 against 1.68 / 3.49).
 int pts_serve_group(const Shape &sh) { return pts_group(sh, 1 << 20); }
 
 // Item of the persistent launch: as many warps as leave room for two CTAs per

@@ -45,10 +45,14 @@
 // per SM a team of warps shares the chain (project_samples).
 //
 // Before, threads owned two time stamps of a sample, evaluated all their rows in
-// every iteration and met at a CTA barrier; per pass, before -> after: 2-D clutter
+// every iteration and met at a CTA barrier; per pass, before -> now: 2-D clutter
 // (N = 1000, n_p = 100, 100 obstacles, K = 100) 195 -> 123 us, 64 uneven 2-D
-// problems (K = 60) 4,534 -> 1,639 us, 3-D ellipsoids (N = 2000, n_p = 150, 200
-// obstacles, K = 100) 826 -> 583 us, a replan of 110 samples (K = 50) 123 -> 102.
+// problems (K = 60) 4,534 -> 1,585 us, 3-D ellipsoids (N = 2000, n_p = 150, 200
+// obstacles, K = 100) 826 -> 492 us, a replan of 110 samples (K = 50) 123 -> 101.
+// Slower than before: samples that keep velocity rows or many pairs active (an iteration
+// of 1,700 cycles, plus 300 a block of rows, 320 a trip of 32 pairs, 5,000 and more a
+// rebuild): 27 circles on a diagonal, 574 samples, K = 75, 220 us against 179; 9 moving
+// circles, 36 samples, K = 92, 220 against 200; 16 circles, 1,520 samples, 170 against 148.
 //
 // The multipliers of the fixed columns (returned only on request) follow from
 // the linearity of eq. lag: lambda_B^K = lambda_B^0 - rho sum_k P_B^T r^k, so
