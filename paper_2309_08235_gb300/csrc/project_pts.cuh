@@ -1022,8 +1022,9 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     const float rho = p.rho, vmax = p.vmax, amax = p.amax;
     const int K = p.K;
     const bool bounds = p.use_bounds != 0, lists = p.list_on != 0;
-    // the obstacles' margin; without obstacles any positive length serves the other rows
-    const float delta = p.list_delta > 0.f ? p.list_delta : 0.01f * vmax * smem()[hdr(kTv) + n_p - 1];
+    // the obstacles' margin; without obstacles any positive length serves the other rows (finite:
+    // margins are halved until they are below a share of it)
+    const float delta = fminf(p.list_delta > 0.f ? p.list_delta : 0.01f * vmax * smem()[hdr(kTv) + n_p - 1], FLT_MAX);
     const int nblk = np / (2 * G);  // blocks of two time stamps per lane (at most 8)
     auto load_node = [&](int i, float2 (&node)[NF + 1]) {
 #pragma unroll
@@ -1110,7 +1111,8 @@ __device__ __forceinline__ void project_samples(const ProjParams<float> &p, int 
     // overflowed built two or three lists a rebuild: 14 moving circles, 574 samples, K = 75,
     // 341 us a pass against 266; 45, 400 samples, K = 60, 625 against 379.)
     float reach = delta;
-    float widest = hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta;
+    float widest =
+        fminf(hdr(kGrid) && __float_as_int(smem()[hdr(kGrid) + 4]) > 0 ? smem()[hdr(kGrid) + 7] : 8.f * delta, FLT_MAX);
     int built = -kShortLived;
     auto rebuild = [&](int need, int k) {
         const bool need_p = need & 1, need_a = need & 2;

@@ -113,3 +113,17 @@ def test_default_margin_changes_no_bit(P, oracle):  # noqa: F811
         same(got, project(P, p, xi, 40, lam0, "1"))
     finally:
         os.environ.pop("PRIEST_LIST_MARGIN")
+
+
+@SHAPES
+@FORMS
+def test_margin_beyond_range(P, oracle, form, dims, mask):  # noqa: F811
+    """Semi-axes whose margin overflows FP32, every pair near: the lists overflow at
+    every margin, and halving it ends."""
+    p = scene(dims=dims, n_obs=40, n_dyn=4, n_p=60, mask=mask)
+    p = dict(p, semi=np.full((40, 2), 2e38))
+    n = PER_SM[form] * sm_count() - 3
+    xi = samples(oracle, p, n, seed=3)
+    got = project(P, p, xi, 8, None, "1")
+    assert got[0].shape == xi.shape
+    same(got, project(P, p, xi, 8, None, "0"))
