@@ -95,7 +95,7 @@ bool pts_allowed()
 // launches would stall a replanner in the middle of its run, or break its capture.
 bool pts_crowded(const Shape &sh, int samples_per_sm)
 {
-    if (!pts_supported(sh) || sh.dims != 2 || sh.n_static >= kGridMinStatic || sh.n_obs < 12) return false;
+    if (!pts_allowed() || !pts_supported(sh) || sh.dims != 2 || sh.n_static >= kGridMinStatic || sh.n_obs < 12) return false;
     double d2 = 0.0;
     for (int ax = 0; ax < sh.dims; ++ax) d2 += (sh.bf[ax][0] - sh.b0[ax][0]) * (sh.bf[ax][0] - sh.b0[ax][0]);
     const bool hurried = std::sqrt(d2) > 0.85 * sh.vmax * sh.horizon;
