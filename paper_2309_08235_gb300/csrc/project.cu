@@ -128,17 +128,26 @@ Tiling choose_tiling(const Shape &sh, int n_samples, int n_sm)
         if (own.smem > 0 && !crowded) return own;
     }
     Tiling t;
-    t.R = sizeof(Real) == 8 || crowded ? 4 : 5;  // (crowded: 141 against 174 us with 5, 33 circles, 110 samples)
+    t.R = sizeof(Real) == 8 ? 4 : 5;
     t.threads = sizeof(Real) == 8 ? 256 : 512;
     const int S0 = m;
     t.ws = 1;
     while (t.ws < 8 && S0 * 32 * (2 * t.ws) <= t.threads && S0 <= 15) t.ws *= 2;
     int S = samples_per_cta(n_samples, n_sm, t.threads, t.ws);
     while (S > 1 && project_smem_bytes<Real>(sh, S, 1) > kSmemCap) S = std::max(1, S * 3 / 4);
-    const int ng = lane_groups<Real>(sh.n_p, t.R);
-    int C = std::max(1, (32 * t.ws) / ng);
-    C = std::min(C, std::max(1, std::min(16, sh.n_obs)));
+    auto chunks = [&](int R) { return std::max(1, (32 * t.ws) / lane_groups<Real>(sh.n_p, R)); };
+    // crowded: four points an item, unless five fill the lanes better (33 circles, K = 50: 110 samples of
+    // 80 stamps 141 against 174 us with five, 1,200 of 150 stamps 315 against 288)
+    if (crowded && 5 * lane_groups<Real>(sh.n_p, 5) * chunks(5) <= 6 * lane_groups<Real>(sh.n_p, 4) * chunks(4)) t.R = 4;
+    int C = std::min(chunks(t.R), std::max(1, std::min(16, sh.n_obs)));
     while (C > 1 && project_smem_bytes<Real>(sh, S, C) > kSmemCap) --C;
+    if (crowded) {
+        // no more chunks than their obstacle pairs need, each costs its partial sums (20 circles,
+        // 300 samples 163 -> 152 us)
+        auto pairs = [](int n, int c) { return (n + 2 * c - 1) / (2 * c); };
+        const int n_mov = sh.n_obs - sh.n_static;
+        while (C > 1 && pairs(sh.n_static, C - 1) == pairs(sh.n_static, C) && pairs(n_mov, C - 1) == pairs(n_mov, C)) --C;
+    }
     t.S = S;
     t.C = C;
     t.smem = project_smem_bytes<Real>(sh, S, C);
