@@ -54,8 +54,8 @@ CASES = {
     "many_samples_full": (lambda: traffic(20, 1.1), 1400, True),
     "fast": (lambda: traffic(40, 1.5, vmax=3.0), 300, False),
     "fast_full": (lambda: traffic(40, 2.1, vmax=3.0), 300, True),
-    "few_samples": (lambda: traffic(20, 0.68, vmax=3.0), 140, False),
-    "few_samples_full": (lambda: traffic(20, 0.72, vmax=3.0), 140, True),
+    "few_samples": (lambda: traffic(20, 0.64, vmax=3.0), 140, False),
+    "few_samples_full": (lambda: traffic(20, 0.66, vmax=3.0), 140, True),
     "few_samples_seven": (lambda: traffic(20, 0.97, vmax=3.0, mask=1), 140, False),
     "few_samples_seven_full": (lambda: traffic(20, 1.03, vmax=3.0, mask=1), 140, True),
     "static": (lambda: traffic(40, 1.5, static=16), 300, False),
