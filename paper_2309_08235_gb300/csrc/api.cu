@@ -1248,8 +1248,8 @@ priest_status batch_tiles(priest_ctx *ctx, const std::vector<Shape> &shapes, std
         // crowded problems alone: the chunked kernel, where it holds them all
         size_t total = 0;
         for (const Shape &sh : shapes) total += size_t(sh.N);
-        // (a batch's items hold several samples, so it gives none an SM of its own)
-        const int m = std::max(2, int((total + ctx->n_sm - 1) / ctx->n_sm));
+        // (a batch's items hold several samples: none has a third of an SM to itself)
+        const int m = std::max(4, int((total + ctx->n_sm - 1) / ctx->n_sm));
         bool crowded = true;
         std::vector<Tiling> chunked(n);
         for (int i = 0; i < n && crowded; ++i) {

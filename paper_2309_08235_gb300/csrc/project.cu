@@ -90,29 +90,28 @@ bool pts_allowed()
 //   292 / 212, 0.89 177 / 167 and 279 / 213, 0.8 167 / 167 and 264 / 213, 0.67 145 / 165 and
 //   219 / 213 (share 0.27: 0.89 147 / 146 and 230 / 187, 0.67 130 / 146 and 175 / 192)
 // (circles on a corridor and, at 0.55 of the bound, crossing traffic; chunked times before
-// the tiling's last 2 to 10 %).  With no more samples than SMs the chunked kernel spreads a
-// sample over a whole SM, and is faster from a share of 0.65 on (1.0 with seven columns)
-// whatever the speed (one scene of thirty 5 % slower): 110 samples, 0.55 of the bound, half
-// of the acceleration bound, discs that stay in a 5 x 3 m box or cross it, K = 60:
-//   share 0.69:  16 discs 149 / 157 and 178 / 157, 33 196 / 165 and 229 / 167, 130 348 / 223
-//                and 435 / 232, 260 524 / 299 and 481 / 270
-//   share 1.34:  16 discs 184 / 157 and 235 / 157, 33 261 / 169 and 340 / 167, 130 462 / 243
-//                and 561 / 250, 260 689 / 316 and 541 / 299
-//   share 0.3:   33 161 / 161 and 195 / 157, 66 207 / 184 and 181 / 186
-//   seven columns, share 0.69 277 / 284, 1.1 329 / 290
-// With more samples than that, which kernel is faster at shares of 0.65 to 2 depends on how
-// long the discs stay on the way, which the share of their first box does not tell (1,000
-// samples, share 0.69: 419 / 380 above, 261 / 425 where they cross and leave).  3-D: the
-// point-owner kernel is faster at every share (33 to 200 spheres: 127 to 386 against 186 to
-// 1,021).  The route depends on the obstacles' values, so it takes the model's tiling: trial
-// launches would stall a replanner in the middle of its run, or break its capture.
+// the tiling's last 2 to 10 %).  With at most three samples per SM the chunked kernel spreads
+// each over a third of an SM or more, and from a share of 1.2 on it is the faster one whatever
+// the speed: 0.55 of the bound, half of the acceleration bound, K = 60, 110 and 400 samples:
+//   share 1.3, discs that stay in a 5 x 3 m box:    16 184 / 157 and 254 / 194, 33 261 / 169 and
+//                                       337 / 222, 130 462 / 243 and 661 / 346
+//              that cross it:           16 235 / 157 and 356 / 194, 33 340 / 167 and 454 / 218
+//              that leave it or a 14 x 20 m box: 24 to 120 discs, 0.98 to 2.4 times the chunked time
+//   share 0.7:  those that stay or cross 0.95 to 3.2 times, those that leave 0.74 to 1.6 times
+//   seven columns, share 1.1: 329 / 290 and 436 / 340, 0.69: 277 / 284 and 331 / 336
+// With more samples, what is faster at shares of 1.2 to 2 depends on how long the discs stay
+// on the way, which the share of their first box does not tell (1,000 samples, share 1.3: 0.73 to
+// 2.7 times, 1.9: 1.04 and more).  3-D: the point-owner kernel is faster at every share (33 to
+// 200 spheres: 127 to 386 against 186 to 1,021).  The route depends on the obstacles' values, so
+// it takes the model's tiling: trial launches would stall a replanner in the middle of its run,
+// or break its capture.
 bool pts_crowded(const Shape &sh, int samples_per_sm)
 {
     if (!pts_allowed() || !pts_supported(sh) || sh.dims != 2 || sh.n_static >= kGridMinStatic || sh.n_obs < 12) return false;
     double d2 = 0.0;
     for (int ax = 0; ax < sh.dims; ++ax) d2 += (sh.bf[ax][0] - sh.b0[ax][0]) * (sh.bf[ax][0] - sh.b0[ax][0]);
     const bool hurried = std::sqrt(d2) > 0.85 * sh.vmax * sh.horizon;
-    if (!hurried) return sh.crowd >= (samples_per_sm > 1 ? 2.0 : sh.nf == 5 ? 0.65 : 1.0);
+    if (!hurried) return sh.crowd >= (samples_per_sm > 3 ? 2.0 : 1.2);
     return sh.crowd >= (sh.nf == 5 && samples_per_sm <= 8 ? 0.25 : 1.0);
 }
 

@@ -52,12 +52,12 @@ CASES = {
     "few": (lambda: traffic(11, 0.6), 300, False),
     "many_samples": (lambda: traffic(20, 0.9), 1400, False),
     "many_samples_full": (lambda: traffic(20, 1.1), 1400, True),
-    "fast": (lambda: traffic(40, 1.5, vmax=3.0), 300, False),
-    "fast_full": (lambda: traffic(40, 2.1, vmax=3.0), 300, True),
-    "few_samples": (lambda: traffic(20, 0.64, vmax=3.0), 140, False),
-    "few_samples_full": (lambda: traffic(20, 0.66, vmax=3.0), 140, True),
-    "few_samples_seven": (lambda: traffic(20, 0.97, vmax=3.0, mask=1), 140, False),
-    "few_samples_seven_full": (lambda: traffic(20, 1.03, vmax=3.0, mask=1), 140, True),
+    "fast": (lambda: traffic(40, 1.5, vmax=3.0), 620, False),
+    "fast_full": (lambda: traffic(40, 2.1, vmax=3.0), 620, True),
+    "fast_few": (lambda: traffic(20, 1.17, vmax=3.0), 450, False),
+    "fast_few_full": (lambda: traffic(20, 1.23, vmax=3.0), 450, True),
+    "fast_few_seven": (lambda: traffic(20, 1.17, vmax=3.0, mask=1), 140, False),
+    "fast_few_seven_full": (lambda: traffic(20, 1.23, vmax=3.0, mask=1), 140, True),
     "static": (lambda: traffic(40, 1.5, static=16), 300, False),
     "seven": (lambda: traffic(20, 0.9, mask=1), 300, False),
     "seven_full": (lambda: traffic(20, 1.1, mask=1), 300, True),
